@@ -10,8 +10,7 @@
 //   S3 = sum_nu stap_nu[F];  S5 = sum_rho stap_rho[sum_{nu != rho} stap_nu[F]];
 //   S7 = sum_sig stap_sig[sum_{rho != sig} stap_rho[sum_{nu != rho, sig} stap_nu[F]]];
 //   L  = the staples whose detour is two steps along nu
-// (all directions different from mu).  Everything is FP64.  One thread per (site, mu) builds
-// every path on the fly; the set-up cost is paid once per gauge configuration.
+// (all directions different from mu).  Everything is FP64.
 // The projection uses the scaled Newton iteration for the polar decomposition,
 //   X <- (g X + X^{-+} / g) / 2,  g = (|X^-1|_F / |X|_F)^(1/2)
 // (N. J. Higham, "Computing the polar decomposition - with applications", SIAM J. Sci. Stat.
@@ -29,13 +28,23 @@ struct M3 {
 };
 
 __device__ __forceinline__ double2 cmul(double2 x, double2 y) { return make_double2(x.x * y.x - x.y * y.y, x.x * y.y + x.y * y.x); }
-__device__ __forceinline__ double2 cmulc(double2 x, double2 y) // x * conj(y)
+
+// s += x y, s += x conj(y), s += conj(x) y: four FMAs each.  (A product formed first and then
+// added costs six FP64 operations, and the FP64 pipe is what bounds these kernels.)
+__device__ __forceinline__ void mac(double2 &s, double2 x, double2 y)
 {
-    return make_double2(x.x * y.x + x.y * y.y, x.y * y.x - x.x * y.y);
+    s.x = fma(x.x, y.x, fma(-x.y, y.y, s.x));
+    s.y = fma(x.x, y.y, fma(x.y, y.x, s.y));
 }
-__device__ __forceinline__ double2 ccmul(double2 x, double2 y) // conj(x) * y
+__device__ __forceinline__ void mac_c(double2 &s, double2 x, double2 y)
 {
-    return make_double2(x.x * y.x + x.y * y.y, x.x * y.y - x.y * y.x);
+    s.x = fma(x.x, y.x, fma(x.y, y.y, s.x));
+    s.y = fma(x.y, y.x, fma(-x.x, y.y, s.y));
+}
+__device__ __forceinline__ void cmac(double2 &s, double2 x, double2 y)
+{
+    s.x = fma(x.x, y.x, fma(x.y, y.y, s.x));
+    s.y = fma(x.x, y.y, fma(-x.y, y.x, s.y));
 }
 
 __device__ __forceinline__ M3 zero()
@@ -47,7 +56,7 @@ __device__ __forceinline__ M3 zero()
 }
 
 // A B, A B^+, A^+ B
-__device__ M3 mul(const M3 &A, const M3 &B)
+__device__ __forceinline__ M3 mul(const M3 &A, const M3 &B)
 {
     M3 r;
 #pragma unroll
@@ -56,16 +65,12 @@ __device__ M3 mul(const M3 &A, const M3 &B)
         for (int k = 0; k < 3; k++) {
             double2 s = make_double2(0.0, 0.0);
 #pragma unroll
-            for (int j = 0; j < 3; j++) {
-                const double2 p = cmul(A.a[3 * i + j], B.a[3 * j + k]);
-                s.x += p.x;
-                s.y += p.y;
-            }
+            for (int j = 0; j < 3; j++) mac(s, A.a[3 * i + j], B.a[3 * j + k]);
             r.a[3 * i + k] = s;
         }
     return r;
 }
-__device__ M3 mul_d(const M3 &A, const M3 &B)
+__device__ __forceinline__ M3 mul_d(const M3 &A, const M3 &B)
 {
     M3 r;
 #pragma unroll
@@ -74,16 +79,12 @@ __device__ M3 mul_d(const M3 &A, const M3 &B)
         for (int k = 0; k < 3; k++) {
             double2 s = make_double2(0.0, 0.0);
 #pragma unroll
-            for (int j = 0; j < 3; j++) {
-                const double2 p = cmulc(A.a[3 * i + j], B.a[3 * k + j]);
-                s.x += p.x;
-                s.y += p.y;
-            }
+            for (int j = 0; j < 3; j++) mac_c(s, A.a[3 * i + j], B.a[3 * k + j]);
             r.a[3 * i + k] = s;
         }
     return r;
 }
-__device__ M3 d_mul(const M3 &A, const M3 &B)
+__device__ __forceinline__ M3 d_mul(const M3 &A, const M3 &B)
 {
     M3 r;
 #pragma unroll
@@ -92,11 +93,7 @@ __device__ M3 d_mul(const M3 &A, const M3 &B)
         for (int k = 0; k < 3; k++) {
             double2 s = make_double2(0.0, 0.0);
 #pragma unroll
-            for (int j = 0; j < 3; j++) {
-                const double2 p = ccmul(A.a[3 * j + i], B.a[3 * j + k]);
-                s.x += p.x;
-                s.y += p.y;
-            }
+            for (int j = 0; j < 3; j++) cmac(s, A.a[3 * j + i], B.a[3 * j + k]);
             r.a[3 * i + k] = s;
         }
     return r;
@@ -115,124 +112,180 @@ struct Lat {
     uint32_t V, Vh;
 };
 
+// Coordinates of canonical site i (even sites first, each parity in lexicographic order), so that
+// consecutive threads read and write consecutive 144-byte records.
+__device__ __forceinline__ void coords(const Lat &L, uint32_t i, int (&c)[4])
+{
+    const uint32_t p = i >= L.Vh;
+    uint32_t q = i - p * L.Vh;
+    const uint32_t nxh = (uint32_t)L.n[0] / 2;
+    const uint32_t xh = q % nxh;
+    q /= nxh;
+    c[1] = (int)(q % (uint32_t)L.n[1]);
+    q /= (uint32_t)L.n[1];
+    c[2] = (int)(q % (uint32_t)L.n[2]);
+    c[3] = (int)(q / (uint32_t)L.n[2]);
+    c[0] = (int)(2 * xh + ((p + c[1] + c[2] + c[3]) & 1));
+}
+
 __device__ __forceinline__ uint32_t site_index(const Lat &L, const int (&c)[4])
 {
-    const uint32_t lex = (uint32_t)(c[0] + L.n[0] * (c[1] + L.n[1] * (c[2] + L.n[2] * c[3])));
+    const uint32_t lex = (uint32_t)c[0] + (uint32_t)L.n[0] * ((uint32_t)c[1] + (uint32_t)L.n[1] * ((uint32_t)c[2] + (uint32_t)L.n[2] * (uint32_t)c[3]));
     return (lex >> 1) + L.Vh * (uint32_t)((c[0] + c[1] + c[2] + c[3]) & 1);
 }
 
-// the link of direction mu at the site c + k * hat(d) (periodic)
-__device__ __forceinline__ M3 load(const Lat &L, const double2 *f, int mu, const int (&c)[4], int d = 0, int k = 0,
-                                   int d2 = 0, int k2 = 0)
-{
-    int y[4] = {c[0], c[1], c[2], c[3]};
-    y[d] = ((y[d] + k) % L.n[d] + L.n[d]) % L.n[d];
-    y[d2] = ((y[d2] + k2) % L.n[d2] + L.n[d2]) % L.n[d2];
-    const double2 *p = f + ((size_t)mu * L.V + site_index(L, y)) * 9;
-    M3 r;
-#pragma unroll
-    for (int i = 0; i < 9; i++) r.a[i] = __ldg(p + i);
-    return r;
-}
-
+// one step along d, forward (k = 1) or backward (k = -1), periodic
 __device__ __forceinline__ void move(const Lat &L, int (&y)[4], int d, int k)
 {
-    y[d] = ((y[d] + k) % L.n[d] + L.n[d]) % L.n[d];
+#pragma unroll
+    for (int e = 0; e < 4; e++)
+        if (e == d) {
+            y[e] += k;
+            if (y[e] == L.n[e]) y[e] = 0;
+            if (y[e] < 0) y[e] += L.n[e];
+        }
 }
 
-// stap_nu[F]_mu(y), F = the field f of direction mu, links u
-__device__ M3 stap1(const Lat &L, const double2 *u, const double2 *f, int mu, int nu, const int (&y)[4])
+// index of the site one step from c along d, and of the one a further step along d2
+__device__ __forceinline__ uint32_t at(const Lat &L, const int (&c)[4], int d, int k)
 {
-    // U_nu(y) F(y+nu) U_nu(y+mu)^+
-    M3 r = mul_d(mul(load(L, u, nu, y), load(L, f, mu, y, nu, 1)), load(L, u, nu, y, mu, 1));
-    // U_nu(y-nu)^+ F(y-nu) U_nu(y-nu+mu)
-    const M3 b = mul(d_mul(load(L, u, nu, y, nu, -1), load(L, f, mu, y, nu, -1)), load(L, u, nu, y, nu, -1, mu, 1));
-    axpy(r, 1.0, b);
-    return r;
+    int y[4] = {c[0], c[1], c[2], c[3]};
+    move(L, y, d, k);
+    return site_index(L, y);
+}
+__device__ __forceinline__ uint32_t at(const Lat &L, const int (&c)[4], int d, int k, int d2, int k2)
+{
+    int y[4] = {c[0], c[1], c[2], c[3]};
+    move(L, y, d, k);
+    move(L, y, d2, k2);
+    return site_index(L, y);
 }
 
-// stap_rho[stap_nu[F]]_mu(y)
-__device__ M3 stap2(const Lat &L, const double2 *u, const double2 *f, int mu, int rho, int nu, const int (&y)[4])
+// matrix i of a field of V matrices (coherent loads: a launch may read what the one before wrote)
+__device__ __forceinline__ M3 load(const double2 *f, size_t i)
 {
-    int yp[4] = {y[0], y[1], y[2], y[3]}, ym[4] = {y[0], y[1], y[2], y[3]};
-    move(L, yp, rho, 1);
-    move(L, ym, rho, -1);
-    M3 r = mul_d(mul(load(L, u, rho, y), stap1(L, u, f, mu, nu, yp)), load(L, u, rho, y, mu, 1));
-    const M3 b = mul(d_mul(load(L, u, rho, y, rho, -1), stap1(L, u, f, mu, nu, ym)), load(L, u, rho, ym, mu, 1));
-    axpy(r, 1.0, b);
+    const double2 *p = f + i * 9;
+    M3 r;
+#pragma unroll
+    for (int k = 0; k < 9; k++) r.a[k] = p[k];
     return r;
 }
-
-// stap_sig[stap_rho[stap_nu[F]]]_mu(y)
-__device__ M3 stap3(const Lat &L, const double2 *u, const double2 *f, int mu, int sig, int rho, int nu, const int (&y)[4])
+__device__ __forceinline__ void store(double2 *f, size_t i, const M3 &m)
 {
-    int yp[4] = {y[0], y[1], y[2], y[3]}, ym[4] = {y[0], y[1], y[2], y[3]};
-    move(L, yp, sig, 1);
-    move(L, ym, sig, -1);
-    M3 r = mul_d(mul(load(L, u, sig, y), stap2(L, u, f, mu, rho, nu, yp)), load(L, u, sig, y, mu, 1));
-    const M3 b = mul(d_mul(load(L, u, sig, y, sig, -1), stap2(L, u, f, mu, rho, nu, ym)), load(L, u, sig, ym, mu, 1));
-    axpy(r, 1.0, b);
-    return r;
+    double2 *p = f + i * 9;
+#pragma unroll
+    for (int k = 0; k < 9; k++) p[k] = m.a[k];
 }
 
-// the staple whose detour is two steps along nu
-__device__ M3 lepage(const Lat &L, const double2 *u, const double2 *f, int mu, int nu, const int (&y)[4])
+// The two halves of stap_nu[F]_mu(x) = up + down for a field of V matrices F (of direction mu):
+//   up   = U_nu(x) F(x+nu) U_nu(x+mu)^+,   down = U_nu(x-nu)^+ F(x-nu) U_nu(x-nu+mu)
+// with Fu, Fd the matrices F(x+nu), F(x-nu).
+__device__ __forceinline__ M3 stap_up(const Lat &L, const double2 *u, int mu, int nu, const int (&x)[4], const M3 &Fu)
 {
-    // U_nu(y) U_nu(y+nu) F(y+2nu) [U_nu(y+mu) U_nu(y+mu+nu)]^+
-    const M3 up = mul(load(L, u, nu, y), load(L, u, nu, y, nu, 1));
-    const M3 upm = mul(load(L, u, nu, y, mu, 1), load(L, u, nu, y, mu, 1, nu, 1));
-    M3 r = mul_d(mul(up, load(L, f, mu, y, nu, 2)), upm);
-    // [U_nu(y-2nu) U_nu(y-nu)]^+ F(y-2nu) U_nu(y-2nu+mu) U_nu(y-nu+mu)
-    const M3 dn = mul(load(L, u, nu, y, nu, -2), load(L, u, nu, y, nu, -1));
-    const M3 dnm = mul(load(L, u, nu, y, nu, -2, mu, 1), load(L, u, nu, y, nu, -1, mu, 1));
-    axpy(r, 1.0, mul(d_mul(dn, load(L, f, mu, y, nu, -2)), dnm));
-    return r;
+    const size_t o = (size_t)nu * L.V;
+    return mul_d(mul(load(u, o + site_index(L, x)), Fu), load(u, o + at(L, x, mu, 1)));
+}
+__device__ __forceinline__ M3 stap_down(const Lat &L, const double2 *u, int mu, int nu, const int (&x)[4], const M3 &Fd)
+{
+    const size_t o = (size_t)nu * L.V;
+    return mul(d_mul(load(u, o + at(L, x, nu, -1)), Fd), load(u, o + at(L, x, nu, -1, mu, 1)));
 }
 
 struct Coef {
     double c1, c3, c5, c7, cl;
 };
 
-// out_mu(x) = c1 F + c3 S3 + c5 S5 + c7 S7 + cl L, one thread per (site, mu)
-__global__ void __launch_bounds__(64) k_smear_level(Lat L, const double2 *u, const double2 *f, double2 *out, Coef c)
+// One level for one direction mu, in three launches over the sites.  The nested staples are built
+// from each other, with every intermediate stored:
+//   1  T_nu = stap_nu[F], its halves apart when Lepage paths are wanted
+//   2  G_rho = c5 sum_{nu != rho} T_nu + c7 (stap_a[T_b] + stap_b[T_a]),  {a, b} = not mu, rho
+//   3  out = c1 F + c3 sum T + sum_rho stap_rho[G_rho] (+ Lepage)
+// A Lepage path is the upper half around an upper half, or the lower around a lower, along one
+// direction, so launch 3 only adds cl T_up to what the upper half encloses and cl T_down to the
+// lower: no product of its own.  48 matrix products per link and level; building every path from
+// its links took 252 (300 with Lepage).
+// FP64-bound (48 x 108 FMAs per link at two a clock and SM): one thread per (site, detour) in
+// launches 1 and 2, one per site in 3, all with consecutive sites in consecutive lanes.
+// 24^3 x 8, the whole call with projection and Naik links: 76.0 ms before, 12.4 ms now (7.7 ms
+// is what the FP64 pipe needs for the products).
+__global__ void __launch_bounds__(128) k_stap3(Lat L, const double2 *u, int mu, double2 *t, double2 *td)
 {
-    const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    if (t >= 4ull * L.V) return;
-    const int mu = (int)(t / L.V);
-    uint32_t lex = (uint32_t)(t - (uint64_t)mu * L.V);
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= L.V) return;
+    const int n = blockIdx.y, nu = n + (n >= mu);
     int x[4];
-#pragma unroll
-    for (int d = 0; d < 4; d++) {
-        x[d] = (int)(lex % (uint32_t)L.n[d]);
-        lex /= (uint32_t)L.n[d];
-    }
+    coords(L, i, x);
+    const double2 *f = u + (size_t)mu * L.V * 9;
+    M3 up = stap_up(L, u, mu, nu, x, load(f, at(L, x, nu, 1)));
+    const M3 dn = stap_down(L, u, mu, nu, x, load(f, at(L, x, nu, -1)));
+    if (td) store(td, (size_t)n * L.V + i, dn);
+    else axpy(up, 1.0, dn);
+    store(t, (size_t)n * L.V + i, up);
+}
+
+// T_n at site j (its halves added when they are stored apart)
+__device__ __forceinline__ M3 load_t(const Lat &L, const double2 *t, const double2 *td, int n, uint32_t j)
+{
+    M3 r = load(t, (size_t)n * L.V + j);
+    if (td) axpy(r, 1.0, load(td, (size_t)n * L.V + j));
+    return r;
+}
+
+__global__ void __launch_bounds__(128) k_stap5(Lat L, const double2 *u, int mu, const double2 *t, const double2 *td,
+                                               double2 *g, Coef c)
+{
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= L.V) return;
+    const int n = blockIdx.y; // rho, as the n-th direction other than mu
+    int x[4];
+    coords(L, i, x);
     M3 acc = zero();
-    axpy(acc, c.c1, load(L, f, mu, x));
-    for (int nu = 0; nu < 4; nu++) {
-        if (nu == mu) continue;
-        axpy(acc, c.c3, stap1(L, u, f, mu, nu, x));
-        if (c.cl != 0.0) axpy(acc, c.cl, lepage(L, u, f, mu, nu, x));
+#pragma unroll 1
+    for (int k = 1; k < 3; k++) {
+        const int na = (n + k) % 3, nb = (n + 3 - k) % 3; // the two other detours, in both orders
+        const int a = na + (na >= mu);
+        axpy(acc, c.c7, stap_up(L, u, mu, a, x, load_t(L, t, td, nb, at(L, x, a, 1))));
+        axpy(acc, c.c7, stap_down(L, u, mu, a, x, load_t(L, t, td, nb, at(L, x, a, -1))));
+        axpy(acc, c.c5, load_t(L, t, td, na, i));
     }
-    for (int rho = 0; rho < 4; rho++) {
-        if (rho == mu) continue;
-        for (int nu = 0; nu < 4; nu++) {
-            if (nu == mu || nu == rho) continue;
-            axpy(acc, c.c5, stap2(L, u, f, mu, rho, nu, x));
-        }
+    store(g, (size_t)n * L.V + i, acc);
+}
+
+__global__ void __launch_bounds__(128) k_stap7(Lat L, const double2 *u, int mu, const double2 *t, const double2 *td,
+                                               const double2 *g, double2 *out, Coef c)
+{
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= L.V) return;
+    int x[4];
+    coords(L, i, x);
+    M3 acc = zero();
+    axpy(acc, c.c1, load(u, (size_t)mu * L.V + i));
+#pragma unroll 1
+    for (int n = 0; n < 3; n++) {
+        const int rho = n + (n >= mu);
+        const uint32_t ju = at(L, x, rho, 1), jd = at(L, x, rho, -1);
+        M3 F = load(g, (size_t)n * L.V + ju);
+        if (td) axpy(F, c.cl, load(t, (size_t)n * L.V + ju));
+        axpy(acc, 1.0, stap_up(L, u, mu, rho, x, F));
+        F = load(g, (size_t)n * L.V + jd);
+        if (td) axpy(F, c.cl, load(td, (size_t)n * L.V + jd));
+        axpy(acc, 1.0, stap_down(L, u, mu, rho, x, F));
+        axpy(acc, c.c3, load_t(L, t, td, n, i));
     }
-    for (int sig = 0; sig < 4; sig++) {
-        if (sig == mu) continue;
-        for (int rho = 0; rho < 4; rho++) {
-            if (rho == mu || rho == sig) continue;
-            for (int nu = 0; nu < 4; nu++) {
-                if (nu == mu || nu == rho || nu == sig) continue;
-                axpy(acc, c.c7, stap3(L, u, f, mu, sig, rho, nu, x));
-            }
-        }
+    store(out, (size_t)mu * L.V + i, acc);
+}
+
+// One smearing level of the links u into out.  t, td, g: scratch of 3 V matrices each (td NULL: no
+// Lepage paths); none of them overlaps u or out.
+static void smear_level(const Lat &L, const double2 *u, double2 *out, double2 *t, double2 *td, double2 *g, const Coef &c,
+                        cudaStream_t st)
+{
+    const unsigned nb = (L.V + 127) / 128;
+    for (int mu = 0; mu < 4; mu++) {
+        k_stap3<<<dim3(nb, 3), 128, 0, st>>>(L, u, mu, t, td);
+        k_stap5<<<dim3(nb, 3), 128, 0, st>>>(L, u, mu, t, td, g, c);
+        k_stap7<<<nb, 128, 0, st>>>(L, u, mu, t, td, g, out, c);
     }
-    double2 *p = out + ((size_t)mu * L.V + site_index(L, x)) * 9;
-#pragma unroll
-    for (int i = 0; i < 9; i++) p[i] = acc.a[i];
 }
 
 // inverse of a 3x3 complex matrix by cofactors; returns false if singular
@@ -319,20 +372,16 @@ __global__ void __launch_bounds__(128) k_project_u3(const double2 *v, double2 *w
 // N_mu(x) = cN W_mu(x) W_mu(x+mu) W_mu(x+2mu)
 __global__ void __launch_bounds__(128) k_naik(Lat L, const double2 *w, double2 *out, double cn)
 {
-    const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    if (t >= 4ull * L.V) return;
-    const int mu = (int)(t / L.V);
-    uint32_t lex = (uint32_t)(t - (uint64_t)mu * L.V);
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= L.V) return;
+    const int mu = blockIdx.y;
     int x[4];
-#pragma unroll
-    for (int d = 0; d < 4; d++) {
-        x[d] = (int)(lex % (uint32_t)L.n[d]);
-        lex /= (uint32_t)L.n[d];
-    }
-    const M3 r = mul(mul(load(L, w, mu, x), load(L, w, mu, x, mu, 1)), load(L, w, mu, x, mu, 2));
-    double2 *p = out + ((size_t)mu * L.V + site_index(L, x)) * 9;
-#pragma unroll
-    for (int i = 0; i < 9; i++) p[i] = make_double2(cn * r.a[i].x, cn * r.a[i].y);
+    coords(L, i, x);
+    const double2 *f = w + (size_t)mu * L.V * 9;
+    const M3 r = mul(mul(load(f, i), load(f, at(L, x, mu, 1))), load(f, at(L, x, mu, 1, mu, 1)));
+    M3 o = zero();
+    axpy(o, cn, r);
+    store(out, (size_t)mu * L.V + i, o);
 }
 
 }  // namespace smear
@@ -375,12 +424,14 @@ extern "C" int hisq_smear_links(const int dims[4], const double *thin, double *f
     cudaError_t e = cudaMemsetAsync(status, 0, sizeof(DevStatus), st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(u, thin, bytes, links_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st);
-    const unsigned nb64 = (unsigned)((4 * V + 63) / 64), nb128 = (unsigned)((4 * V + 127) / 128);
+    const unsigned nb = (unsigned)((V + 127) / 128), nb4 = (unsigned)((4 * V + 127) / 128);
     if (e == cudaSuccess) {
-        smear::k_smear_level<<<nb64, 64, 0, st>>>(L, u, u, v, smear::Coef{1.0 / 8, 1.0 / 16, 1.0 / 64, 1.0 / 384, 0.0});
-        smear::k_project_u3<<<nb128, 128, 0, st>>>(v, w, 4 * V, status);
-        smear::k_smear_level<<<nb64, 64, 0, st>>>(L, w, w, xo, smear::Coef{1.0, 1.0 / 16, 1.0 / 64, 1.0 / 384, -1.0 / 8});
-        smear::k_naik<<<nb128, 128, 0, st>>>(L, w, no, -1.0 / 24 + eps_naik / 8);
+        // scratch of a level (three matrices per site each): fields that hold nothing yet or no
+        // longer, so no memory beyond the links, the two levels and the results is needed
+        smear::smear_level(L, u, v, w, nullptr, xo, smear::Coef{1.0 / 8, 1.0 / 16, 1.0 / 64, 1.0 / 384, 0.0}, st);
+        smear::k_project_u3<<<nb4, 128, 0, st>>>(v, w, 4 * V, status);
+        smear::smear_level(L, w, xo, u, v, no, smear::Coef{1.0, 1.0 / 16, 1.0 / 64, 1.0 / 384, -1.0 / 8}, st);
+        smear::k_naik<<<dim3(nb, 4), 128, 0, st>>>(L, w, no, -1.0 / 24 + eps_naik / 8);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && !links_on_device) {

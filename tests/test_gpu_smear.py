@@ -30,6 +30,17 @@ def test_smeared_links_match_oracle(dims, eps_naik):
     assert torch.equal(fh, fat.cpu()) and torch.equal(lh, lng.cpu())
 
 
+@pytest.mark.parametrize("dims", [(10, 4, 6, 4), (4, 4, 4, 6), (6, 14, 4, 10)])
+def test_nested_staples_at_ragged_sizes(dims):
+    # volumes that leave a partly filled last block, extents at which a path wraps around; the
+    # tolerance is the one of the other sizes (FP64 sums of order-one products on both sides)
+    thin, _ = fields.recipe_links(dims, 0.8, 1202)
+    fat, lng = hisq.smear_links(dims, thin.cuda(), eps_naik=-0.2)
+    want_fat, want_lng = smear.hisq_links(dims, thin.numpy(), eps_naik=-0.2)
+    assert np.abs(fat.cpu().numpy() - want_fat).max() <= 1e-13
+    assert np.abs(lng.cpu().numpy() - want_lng).max() <= 1e-14
+
+
 def test_unit_links_give_free_field_links():
     dims = (4, 4, 6, 4)
     vol = int(np.prod(dims))
