@@ -36,9 +36,28 @@ def test_nested_staples_at_ragged_sizes(dims):
     # tolerance is the one of the other sizes (FP64 sums of order-one products on both sides)
     thin, _ = fields.recipe_links(dims, 0.8, 1202)
     fat, lng = hisq.smear_links(dims, thin.cuda(), eps_naik=-0.2)
-    want_fat, want_lng = smear.hisq_links(dims, thin.numpy(), eps_naik=-0.2)
+    want_fat, want_lng = _links_extended(dims, thin.numpy(), -0.2)
     assert np.abs(fat.cpu().numpy() - want_fat).max() <= 1e-13
     assert np.abs(lng.cpu().numpy() - want_lng).max() <= 1e-14
+
+
+def _links_extended(dims, thin, eps_naik):
+    """The oracle's links with the staples and the projection in extended precision: among links this
+    far from unity some smeared ones have a condition number near 100, whose square in V^+ V costs
+    the oracle's FP64 eigendecomposition 1e-13 by itself."""
+    u = smear.to_4d(dims, thin).astype(np.clongdouble)
+    x = smear.smear_level(u, u, **smear.LEVEL1)
+    for _ in range(40):  # Newton iteration for the unitary polar factor: x <- (x + x^{-+}) / 2
+        cof = np.empty_like(x)
+        for i in range(3):
+            for j in range(3):
+                i1, i2, j1, j2 = (i + 1) % 3, (i + 2) % 3, (j + 1) % 3, (j + 2) % 3
+                cof[..., i, j] = x[..., i1, j1] * x[..., i2, j2] - x[..., i1, j2] * x[..., i2, j1]
+        det = (x[..., 0, :] * cof[..., 0, :]).sum(-1)
+        x = (x + np.conj(cof / det[..., None, None])) / 2
+    lng = [(-1 / 24 + eps_naik / 8) * smear.mm(smear.mm(x[mu], smear.shift(x[mu], mu, 1)), smear.shift(x[mu], mu, 2))
+           for mu in range(4)]
+    return smear.from_4d(dims, smear.smear_level(x, x, **smear.LEVEL2)), smear.from_4d(dims, np.stack(lng))
 
 
 def test_unit_links_give_free_field_links():
