@@ -15,6 +15,7 @@
 
 #include "arith.cuh"
 #include "dslash.cuh"
+#include "fixed.cuh"
 
 namespace hisq {
 
@@ -85,6 +86,7 @@ struct ImportArgs {
     char *base;
     size_t slot_bytes;
     int prec, nreal, phased;
+    int fixed; // FP64 with 18 reals: the fixed-point words of fixed.cuh instead of doubles
     double inv_scale[2];  // stored = sign * link * inv_scale
 };
 
@@ -106,7 +108,11 @@ __global__ void k_import_links(const ImportArgs a)
         const double sg = (neg ? -1.0 : 1.0) * a.inv_scale[type];
         const size_t V = 2ull * a.g.Vh;
         const double *L = a.src[type] + ((size_t)mu * V + (size_t)p * a.g.Vh + s) * 18;
-        for (int i = 0; i < a.nreal; i++) {
+        if (a.fixed) {
+            double d[18];
+            for (int i = 0; i < 18; i++) d[i] = sg * L[i];
+            fx_encode_link(d, w);
+        } else for (int i = 0; i < a.nreal; i++) {
             const double d = sg * L[i];
             switch (a.prec) {
             case HISQ_F64: {
@@ -275,6 +281,7 @@ static int build_store(hisq_ctx *ctx, int prec, int nreal, const double *fat, co
     a.prec = prec;
     a.nreal = nreal;
     a.phased = ctx->links_phased;
+    a.fixed = prec == HISQ_F64 && nreal == 18 && !ctx->links_double;
     for (int t = 0; t < 2; t++) {
         double sc = 1.0;
         if (nreal == 12) sc = c[t];
@@ -345,6 +352,14 @@ void hisq_destroy(hisq_ctx *ctx)
 
 int hisq_create(hisq_ctx **out, const int dims[4], const double *fat, const double *lng, const hisq_opts *opts_in)
 {
+    return create_context(out, dims, fat, lng, opts_in, false);
+}
+
+}  // extern "C"
+
+int hisq::create_context(hisq_ctx **out, const int dims[4], const double *fat, const double *lng,
+                         const hisq_opts *opts_in, bool links_double)
+{
     if (!out) return HISQ_EINVAL;
     *out = nullptr;
     if (!dims || !fat || !lng) return HISQ_EINVAL;
@@ -370,6 +385,7 @@ int hisq_create(hisq_ctx **out, const int dims[4], const double *fat, const doub
     hisq_ctx *ctx = new hisq_ctx();
     ctx->device = opts.device;
     ctx->links_phased = opts.links_phased;
+    ctx->links_double = links_double;
     ctx->autotune = opts.autotune;
     for (int i = 0; i < 4; i++) ctx->dims[i] = dims[i];
     cudaError_t e = cudaSetDevice(opts.device);
@@ -482,6 +498,8 @@ fail:
     hisq_destroy(ctx);
     return rc;
 }
+
+extern "C" {
 
 // ---------------------------------------------------------------- fields
 int hisq_field_create(hisq_ctx *ctx, int prec, int nrhs, hisq_field **f)

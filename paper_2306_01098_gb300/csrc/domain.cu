@@ -267,7 +267,7 @@ int hisq_dd_create(hisq_dd **out, const int gdims[4], int t0, int lt, const doub
         so.device = opts.device;
         so.autotune = 0;
         const int ldims[4] = {gdims[0], gdims[1], gdims[2], lt};
-        rc = hisq_create(&dd->slab, ldims, lf, ll, &so);
+        rc = create_context(&dd->slab, ldims, lf, ll, &so, true); // k_dd_dslash reads doubles
         if (rc) dd_fail(dd, rc, "hisq_dd_create: slab link store");
     }
     if (gf) cudaFree(gf);

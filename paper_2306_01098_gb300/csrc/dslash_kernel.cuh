@@ -25,6 +25,8 @@
 //   * Links (PL) stream through with L1-bypassing 16-byte loads, read once per application;
 //     neighbour spinors (PV) are gathered through L1/L2, where their 16-fold reuse happens.
 //     PL and PV differ only for 16-bit links with FP32 vectors.
+//   * FP64 with 18 reals runs on integers (fixed.cuh), 1.9 times as fast as FP64 multiply-adds on
+//     this GPU and no less precise; 12 reals stay in FP64 (their third row is rebuilt in it).
 // Optional epilogue (normal operator, Sec. 3.2 applyMdaggM):
 //   EPI = 1: out = m4 * p - D in,   and <p, out> reduced in FP64 per right-hand side;
 //   EPI = 2: the same and also |r|^2, <r, out> and <out, out> (four values per right-hand
@@ -37,6 +39,7 @@
 
 #include "arith.cuh"
 #include "dslash.cuh"
+#include "fixed.cuh"
 #include "reduce.cuh"
 
 namespace hisq {
@@ -109,6 +112,123 @@ __device__ __forceinline__ void vec_load(const char *base, uint32_t s, typename 
     else T::load(base, s, v);
 }
 
+// ---------------------------------------------------------------- FP64 sites in fixed point
+// hop number q2 = 2 mu + type of the site's eight pairs of hops
+struct FxHop {
+    uint32_t w[36];
+    uint32_t sn; // the neighbour the hop comes from
+};
+template <bool BACK>
+__device__ __forceinline__ void fx_hop_issue(const DslashArgs &a, const Geom &g, const char *links, size_t slot_bytes,
+                                             const Site &c, uint32_t s, int q2, bool hint, FxHop &x)
+{
+    const int mu = q2 >> 1, type = q2 & 1, k = type ? 3 : 1;
+    bool wrap;
+    x.sn = neighbour(g, c, s, mu, BACK ? -k : k, wrap);
+    const int lp = BACK ? 1 - a.p : a.p;
+    load_link_words<144>(links + (size_t)((lp * 2 + type) * 4 + mu) * slot_bytes, BACK ? x.sn : s, x.w, hint);
+}
+
+// the hops q2 in [q0, q1) of site s in FP64, one at a time: sites that hold what the fixed-point
+// format cannot (infinities, NaN, extreme magnitudes)
+static __device__ __noinline__ void fx_site_f64(const DslashArgs &a, const Geom &g, const char *links, size_t slot_bytes,
+                                                const char *in, uint32_t s, int q0, int q1, double (&out)[6])
+{
+    const Site c = site_coords(g, s, a.p);
+    for (int i = 0; i < 6; i++) out[i] = 0.0;
+#pragma unroll 1
+    for (int q = 2 * q0; q < 2 * q1; q++) {
+        const int mu = q >> 2, type = (q >> 1) & 1, k = type ? 3 : 1;
+        const bool back = q & 1;
+        bool wrap;
+        const uint32_t sn = neighbour(g, c, s, mu, back ? -k : k, wrap);
+        const int lp = back ? 1 - a.p : a.p;
+        uint32_t w[36];
+        load_link_words<144>(links + (size_t)((lp * 2 + type) * 4 + mu) * slot_bytes, back ? sn : s, w);
+        const uint32_t code = fx_code(w);
+        Prec<HISQ_F64>::Link U;
+        Prec<HISQ_F64>::Vec v;
+        Prec<HISQ_F64>::Acc acc;
+#pragma unroll
+        for (int i = 0; i < 18; i++) U.v[i] = fx_decode(w[2 * i], w[2 * i + 1], code);
+#pragma unroll
+        for (int i = 0; i < 6; i++) acc.v[i] = out[i];
+        Prec<HISQ_F64>::load(in, sn, v);
+        if (back) Prec<HISQ_F64>::hop<true, true>(acc, U, v);
+        else Prec<HISQ_F64>::hop<false, false>(acc, U, v);
+#pragma unroll
+        for (int i = 0; i < 6; i++) out[i] = acc.v[i];
+    }
+}
+
+// D in at site s for NR right-hand sides in fixed point (fixed.cuh), the directions of one of DS
+// threads per site, summed over these threads.
+// The links of the next hop and the vector of the next product are loaded before the current one
+// is worked on: its branches (a larger exponent, a vector of zeros) would keep the compiler from
+// moving the loads there.  The hops are a loop of eight pairs, which keeps the code in the
+// instruction cache.
+template <int NR, int DS>
+__device__ __forceinline__ void fx_site(const DslashArgs &a, const Geom &g, const char *links, size_t slot_bytes,
+                                        const char *in, uint32_t s, bool live, int part,
+                                        Prec<HISQ_F64>::Acc (&out)[NR])
+{
+    constexpr int NQ = 8 / DS;
+    const int q0 = part * NQ;
+    FxAcc acc[NR];
+#pragma unroll
+    for (int r = 0; r < NR; r++) fx_zero(acc[r]);
+    if (live) {
+        const bool hint = NR > 1 && a.stream_links != 0;
+        const Site c = site_coords(g, s, a.p);
+        FxHop fw, bw;
+        FxVec v[2]; // product number parity: the current one and the next
+        fx_hop_issue<false>(a, g, links, slot_bytes, c, s, q0, hint, fw);
+        fx_load(in, fw.sn, v[0]);
+#pragma unroll 1
+        for (int q2 = q0; q2 < q0 + NQ; q2++) {
+            fx_hop_issue<true>(a, g, links, slot_bytes, c, s, q2, hint, bw);
+            uint32_t code = fx_code(fw.w);
+#pragma unroll
+            for (int r = 0; r < NR; r++) {
+                fx_load(in + (r + 1 < NR ? (size_t)(r + 1) * a.rhs_bytes : 0), r + 1 < NR ? fw.sn : bw.sn, v[(r + 1) & 1]);
+                fx_hop<false>(acc[r], fw.w, code, v[r & 1]);
+            }
+            const int qn = q2 + 1 < q0 + NQ ? q2 + 1 : q0; // (the last one is not used)
+            fx_hop_issue<false>(a, g, links, slot_bytes, c, s, qn, hint, fw);
+            code = fx_code(bw.w);
+#pragma unroll
+            for (int r = 0; r < NR; r++) {
+                fx_load(in + (r + 1 < NR ? (size_t)(r + 1) * a.rhs_bytes : 0), r + 1 < NR ? bw.sn : fw.sn,
+                        v[(NR + r + 1) & 1]);
+                fx_hop<true>(acc[r], bw.w, code, v[(NR + r) & 1]);
+            }
+        }
+    }
+    bool bad = false;
+#pragma unroll
+    for (int r = 0; r < NR; r++) {
+        if constexpr (DS > 1) fx_combine<DS>(acc[r]);
+        const double sc = fx_scale(acc[r]);
+#pragma unroll
+        for (int k = 0; k < 6; k++) out[r].v[k] = fx_value(acc[r], k, sc);
+        bad |= acc[r].bad;
+    }
+    if (__any_sync(0xffffffffu, bad)) {
+#pragma unroll
+        for (int r = 0; r < NR; r++) {
+            double o[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+            if (live && acc[r].bad)
+                fx_site_f64(a, g, links, slot_bytes, in + (size_t)r * a.rhs_bytes, s, q0, q0 + NQ, o);
+#pragma unroll
+            for (int k = 0; k < 6; k++) {
+#pragma unroll
+                for (int off = DS / 2; off > 0; off >>= 1) o[k] += __shfl_xor_sync(0xffffffffu, o[k], off);
+                if (acc[r].bad) out[r].v[k] = o[k];
+            }
+        }
+    }
+}
+
 // One work item: the sites of one tile (a.bs threads, DS per site; this thread is
 // number tid of the tile) for the NR right-hand sides whose vectors start at in/out/pv/rv
 // (consecutive right-hand sides a.rhs_bytes apart); geometry g, link store `links`.
@@ -167,7 +287,10 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const Geom &g, 
 #pragma unroll
     for (int r = 0; r < NR; r++) T::zero(out[r]);
 
-    if (live) {
+    // FP64 with 18 reals: in fixed point, summed over the site's threads there
+    constexpr bool FX = PL == HISQ_F64 && NREAL == 18;
+    if constexpr (FX) fx_site<NR, DS>(a, g, links, slot_bytes, in, s, live, part, out);
+    else if (live) {
         const Site c = site_coords(g, s, a.p);
         typename T::Acc acc[TWO ? 2 : 1][NR];
 #pragma unroll
@@ -259,7 +382,7 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const Geom &g, 
         }
     }
     // partial sums of the DS threads of a site meet in every one of them
-    if constexpr (DS > 1) {
+    if constexpr (DS > 1 && !FX) {
 #pragma unroll
         for (int off = DS / 2; off > 0; off >>= 1)
 #pragma unroll

@@ -1,0 +1,261 @@
+// fixed.cuh -- link times colour vector in 60-bit fixed point: the arithmetic of the FP64
+// Dslash with 18-real links.
+//
+// This GPU issues two FP64 operations per clock and SM; the 576 multiply-adds of one Dslash
+// site then take 288 clocks where its bytes take about 100.  Integer multiply-adds
+// (32 x 32 + 64 -> 64 bits) issue many times faster, so the products are formed on integers:
+//   a link is  Lambda 2^(e_L - 59),   Lambda integer, |Lambda| <= 2^60, 2^e_L <= max |entry| < 2^(e_L + 1)
+//   a vector is     N 2^(e_v - 59)    likewise, made from its doubles when it is loaded
+// both kept as two limbs, x = h 2^32 + l with -2^31 <= l < 2^31 and |h| <= 2^28.  A product is
+//   h h' 2^64 + (h l' + l h') 2^32     (l l' is dropped: at most 2^-58 of max |entry| max |v|)
+// i.e. three multiply-adds into two 64-bit sums, H and M.  Bounds: H adds 96 products of at most
+// 2^56 per component and site (16 hops, 3 colours, re and im): < 2^62.6.  M adds 12 products of
+// at most 2^59 per hop, and is folded into H after every hop: < 2^62.6 too.  Nothing is lost in
+// the sums; all hops of a site are aligned to the largest exponent e_L + e_v met so far (H and M
+// are shifted when a larger one comes).
+// Errors of a site, relative to the largest |link| |vector| among its hops: 2^-61 (vector) and
+// 2^-61 (link; 2^-57 for the three entries that carry the exponent) per product, against 2^-53
+// per product and per sum in FP64; the sum is rounded to FP64 once.
+// Measured (max over a field, relative to its largest entry): 2.5e-16 after the normal operator of a
+// 32^3 x 8 lattice, 3.9e-16 with FP64 multiply-adds.  Time there, two Dslash launches: 280.8 us with
+// FP64 multiply-adds (their pipe alone needs 250 us), 147.2 us so (the bytes need 93 us).
+// Sites that meet anything this cannot hold (an infinity or NaN, or values below about 1e-280 or
+// products beyond about 1e+-280) are computed in FP64 instead (fx_site_f64).
+#pragma once
+
+#include "internal.cuh"
+
+namespace hisq {
+
+// Stored link, 18 reals: word 2i the low limb, 2i + 1 the high limb of real i.  The low four bits
+// of the low limbs of reals 0, 1, 2 hold the biased exponent e_L + 1023 (the value is rounded to
+// the nearest one with these bits): 0 for a link of zeros, kFxRaw for one that the format cannot
+// hold, whose words are then the doubles themselves.
+constexpr uint32_t kFxRaw = 0xfff;
+constexpr uint32_t kFxMinExp = 64; // smallest biased exponent of a link or vector in fixed point
+// biased exponents of products (sum of two biased exponents) that the sums are formed with
+constexpr uint32_t kFxELo = 1100, kFxEHi = 3000;
+
+__host__ __device__ inline void fx_encode_link(const double (&d)[18], uint32_t (&w)[36])
+{
+    uint64_t b[18];
+    uint32_t em = 0;
+    bool zero = true;
+    for (int i = 0; i < 18; i++) {
+        union { double d; uint64_t u; } c;
+        c.d = d[i];
+        b[i] = c.u;
+        const uint32_t e = (uint32_t)(b[i] >> 52) & 0x7ffu;
+        em = e > em ? e : em;
+        zero = zero && (b[i] << 1) == 0;
+    }
+    const bool raw = !zero && (em < kFxMinExp || em == 0x7ffu);
+    const uint32_t code = zero ? 0u : raw ? kFxRaw : em;
+    for (int i = 0; i < 18; i++) {
+        const int64_t nib = i < 3 ? (int64_t)((code >> (4 * i)) & 15u) : 0;
+        if (raw) {
+            const uint64_t x = i < 3 ? (b[i] & ~15ull) | (uint64_t)nib : b[i];
+            w[2 * i] = (uint32_t)x;
+            w[2 * i + 1] = (uint32_t)(x >> 32);
+            continue;
+        }
+        // 53-bit magnitude, shifted left by 7 (60 bits) and right by the distance to the
+        // largest exponent, to nearest
+        const uint32_t e = (uint32_t)(b[i] >> 52) & 0x7ffu, s = em - e;
+        int64_t x = 0;
+        if (e != 0 && s < 62) {
+            const int64_t m = (int64_t)(((b[i] & 0xfffffffffffffull) | 0x10000000000000ull) << 7);
+            x = (m + (s ? (int64_t)1 << (s - 1) : 0)) >> s;
+            if (b[i] >> 63) x = -x;
+        }
+        if (i < 3) x = ((x - nib + 8) & ~(int64_t)15) + nib;
+        const int32_t l = (int32_t)(uint32_t)x;
+        w[2 * i] = (uint32_t)l;
+        w[2 * i + 1] = (uint32_t)((x - l) >> 32);
+    }
+}
+
+// biased exponent of a stored link
+__host__ __device__ __forceinline__ uint32_t fx_code(const uint32_t (&w)[36])
+{
+    return (w[0] & 15u) | (w[2] & 15u) << 4 | (w[4] & 15u) << 8;
+}
+
+// the link as doubles (fallback and tests)
+__host__ __device__ inline double fx_decode(uint32_t lo, uint32_t hi, uint32_t code)
+{
+    union { double d; uint64_t u; } c;
+    if (code == kFxRaw) {
+        c.u = (uint64_t)hi << 32 | lo;
+        return c.d;
+    }
+    if (code == 0) return 0.0;
+    // 2^(code - 1023 - 59) as a product of two powers (either may leave the normal range alone)
+    c.u = (uint64_t)code << 52;
+    const double x = (double)((int64_t)(int32_t)hi * 4294967296ll + (int32_t)lo);
+    return x * 1.734723475976807e-18 * c.d; // 2^-59
+}
+
+// running sums of one output vector: component k is (H[k] 2^32 + M[k]) 2^(E - 2046 - 118 + 32)
+// E: largest sum of biased exponents so far; bad: a value that the format cannot hold was met
+struct FxAcc {
+    int64_t H[6], M[6];
+    uint32_t E;
+    bool bad;
+};
+
+__device__ __forceinline__ void fx_zero(FxAcc &a)
+{
+#pragma unroll
+    for (int k = 0; k < 6; k++) a.H[k] = a.M[k] = 0;
+    a.E = kFxELo;
+    a.bad = false;
+}
+
+// sums >>= d (d > 0): H and the 32 bits of M, as one 96-bit number
+__device__ __forceinline__ void fx_shift(FxAcc &a, uint32_t d)
+{
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        const int64_t H = a.H[k];
+        const uint32_t f = (uint32_t)a.M[k];
+        if (d < 32) a.M[k] = (int64_t)__funnelshift_r(f, (uint32_t)H, d);
+        else a.M[k] = (int64_t)(uint32_t)(H >> (d - 32 < 63 ? d - 32 : 63));
+        a.H[k] = H >> (d < 63 ? d : 63);
+    }
+}
+
+// M's carry into H; its low 32 bits stay
+__device__ __forceinline__ void fx_fold(FxAcc &a)
+{
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        a.H[k] += (int64_t)(int32_t)(a.M[k] >> 32);
+        a.M[k] = (int64_t)(uint32_t)a.M[k];
+    }
+}
+
+// one colour vector as its doubles' words (lo, hi)
+struct FxVec {
+    uint32_t lo[6], hi[6];
+};
+
+__device__ __forceinline__ void fx_load(const char *base, uint32_t s, FxVec &v)
+{
+    const uint4 *p = reinterpret_cast<const uint4 *>(base + (size_t)s * 48);
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        const uint4 q = __ldg(p + i);
+        v.lo[2 * i] = q.x;
+        v.hi[2 * i] = q.y;
+        v.lo[2 * i + 1] = q.z;
+        v.hi[2 * i + 1] = q.w;
+    }
+}
+
+// a += U v (BACK = false) or a -= U^+ v (BACK = true); w: the stored link, code: its exponent
+template <bool BACK>
+__device__ __forceinline__ void fx_hop(FxAcc &a, const uint32_t (&w)[36], uint32_t code, const FxVec &v)
+{
+    uint32_t top = 0;
+#pragma unroll
+    for (int k = 0; k < 6; k++) top = max(top, v.hi[k] & 0x7fffffffu);
+    const uint32_t ev = top >> 20, e = code ? code + ev : 0u;
+    if (ev - kFxMinExp >= 0x7ffu - kFxMinExp || e - kFxELo > kFxEHi - kFxELo) {
+        // zeros contribute nothing; anything else here is left to FP64
+        uint32_t any = 0;
+#pragma unroll
+        for (int k = 0; k < 6; k++) any |= (v.hi[k] & 0x7fffffffu) | v.lo[k];
+        a.bad |= any != 0 && (code != 0 || ev == 0x7ffu);
+        return;
+    }
+    if (e > a.E) {
+        fx_shift(a, e - a.E);
+        a.E = e;
+    }
+    const uint32_t t = a.E - code; // the vector's exponent in these sums, >= ev
+    int32_t h[6], l[6], nh[3], nl[3];
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        const uint32_t s = t - ((v.hi[k] >> 20) & 0x7ffu);
+        const uint32_t mh = (v.hi[k] & 0xfffffu) | 0x100000u;
+        uint64_t m = (uint64_t)__funnelshift_l(v.lo[k], mh, 7) << 32 | (v.lo[k] << 7);
+        m = s < 64 ? m >> s : 0ull;
+        const uint32_t sg = (uint32_t)((int32_t)(BACK ? ~v.hi[k] : v.hi[k]) >> 31);
+        const int64_t x = (int64_t)(m ^ ((uint64_t)sg << 32 | sg)) - (int64_t)(int32_t)sg;
+        l[k] = (int32_t)(uint32_t)x;
+        h[k] = (int32_t)(x >> 32) + (int32_t)((uint32_t)l[k] >> 31);
+    }
+    // the component that enters with both signs, negated: im forward, re backward
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+        // (-2^31 has no negative in 32 bits: its limb is -(2^31 - 1), one unit of 2^-60 off)
+        nh[j] = -h[2 * j + (BACK ? 0 : 1)];
+        nl[j] = max(-2147483647, l[2 * j + (BACK ? 0 : 1)]);
+        nl[j] = -nl[j];
+    }
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const int q = BACK ? 3 * j + i : 3 * i + j;
+            const int32_t url = (int32_t)w[4 * q], urh = (int32_t)w[4 * q + 1];
+            const int32_t uil = (int32_t)w[4 * q + 2], uih = (int32_t)w[4 * q + 3];
+            const int r = 2 * j, m = 2 * j + 1;
+            // forward: re += ur vr + ui (-vi), im += ur vi + ui vr
+            // backward (h, l hold -v): re += ur (-vr) + ui (-vi), im += ur (-vi) + ui vr
+            const int32_t ah = BACK ? h[m] : nh[j], al = BACK ? l[m] : nl[j];
+            const int32_t bh = BACK ? nh[j] : h[r], bl = BACK ? nl[j] : l[r];
+            int64_t &Hr = a.H[2 * i], &Hi = a.H[2 * i + 1], &Mr = a.M[2 * i], &Mi = a.M[2 * i + 1];
+            Hr += (int64_t)urh * h[r];
+            Hr += (int64_t)uih * ah;
+            Mr += (int64_t)urh * l[r];
+            Mr += (int64_t)url * h[r];
+            Mr += (int64_t)uih * al;
+            Mr += (int64_t)uil * ah;
+            Hi += (int64_t)urh * h[m];
+            Hi += (int64_t)uih * bh;
+            Mi += (int64_t)urh * l[m];
+            Mi += (int64_t)url * h[m];
+            Mi += (int64_t)uih * bl;
+            Mi += (int64_t)uil * bh;
+        }
+    fx_fold(a);
+}
+
+// sum over the DS lanes that share a site, in every one of them
+template <int DS>
+__device__ __forceinline__ void fx_combine(FxAcc &a)
+{
+#pragma unroll
+    for (int off = DS / 2; off > 0; off >>= 1) {
+        const uint32_t eo = __shfl_xor_sync(0xffffffffu, a.E, off);
+        a.bad |= __shfl_xor_sync(0xffffffffu, (int)a.bad, off) != 0;
+        if (eo > a.E) {
+            fx_shift(a, eo - a.E);
+            a.E = eo;
+        }
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+            a.H[k] += __shfl_xor_sync(0xffffffffu, a.H[k], off);
+            a.M[k] += (int64_t)__shfl_xor_sync(0xffffffffu, (uint32_t)a.M[k], off);
+        }
+        fx_fold(a);
+    }
+}
+
+// component k as a double.  The three words become doubles by the exponent trick (2^52 + x and
+// the like are exact), so this takes four FP64 operations and no conversion.
+__device__ __forceinline__ double fx_value(const FxAcc &a, int k, double scale)
+{
+    const uint32_t f = (uint32_t)a.M[k], lo = (uint32_t)(uint64_t)a.H[k], hi = (uint32_t)((uint64_t)a.H[k] >> 32);
+    const double xh = __hiloint2double(0x45300000, (int)(hi ^ 0x80000000u)); // 2^84 + (hi + 2^31) 2^32
+    const double xl = __hiloint2double(0x43300000, (int)lo);                 // 2^52 + lo
+    const double xf = __hiloint2double(0x41300000, (int)f);                  // 2^20 + f 2^-32
+    // 2^84 + 2^63 + 2^52
+    const double s = __dadd_rn(__dsub_rn(xh, __hiloint2double(0x45300000, (int)0x80100000u)), xl);
+    return __dmul_rn(__dadd_rn(s, __dsub_rn(xf, 1048576.0)), scale);
+}
+__device__ __forceinline__ double fx_scale(const FxAcc &a) { return __hiloint2double((int)((a.E - 2100u + 1023u) << 20), 0); }
+
+}  // namespace hisq

@@ -237,6 +237,7 @@ struct hisq_ctx {
     int dims[4] = {0, 0, 0, 0};
     hisq::Geom g{};
     int links_phased = 0;
+    bool links_double = false; // the FP64 store keeps doubles (a domain's own kernel reads it)
     int autotune = 1;
     std::map<long long, hisq::DslashShape> tune; // autotuned Dslash shapes, keyed by hisq::tune_key
     hisq::LinkStore links[HISQ_NPREC];
@@ -277,6 +278,10 @@ void release_fcg_work(hisq_ctx *ctx);
         cudaError_t e_ = (call);                                  \
         if (e_ != cudaSuccess) return hisq::cuda_error((ctx), e_, #call); \
     } while (0)
+
+// hisq_create; links_double: the 18-real FP64 store holds doubles, not the Dslash's fixed point
+int create_context(hisq_ctx **out, const int dims[4], const double *fat, const double *lng, const hisq_opts *opts_in,
+                   bool links_double);
 
 // launch helpers implemented in the .cu files
 int launch_dslash2(hisq_ctx *ctx, int pl, int pv, int out_parity, const void *in, void *out, int nrhs,
