@@ -129,6 +129,41 @@ __device__ __forceinline__ void load_link_words(const char *slot, uint32_t s, ui
     }
 }
 
+// ---------------------------------------------------------------- asynchronous copies to shared memory
+// 16, 8 or 4 bytes each; L1 = false takes 16-byte copies past L1
+template <int N, bool L1>
+__device__ __forceinline__ void cp_async(uint32_t dst, const void *src)
+{
+    if constexpr (N == 16 && !L1) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(N) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// this thread's B bytes in a block's stage: 16-byte chunk q of thread t at q * 16 n + 16 t (n threads),
+// then the 8- or 4-byte tails
+template <int B>
+__device__ __forceinline__ void stage_read(const char *st, uint32_t n, uint32_t t, uint32_t (&w)[B / 4])
+{
+    constexpr int NQ = B / 16, TB = B % 16;
+#pragma unroll
+    for (int q = 0; q < NQ; q++) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(st + (size_t)(q * n + t) * 16);
+        w[4 * q] = v.x;
+        w[4 * q + 1] = v.y;
+        w[4 * q + 2] = v.z;
+        w[4 * q + 3] = v.w;
+    }
+    if constexpr (TB == 8) {
+        const uint2 v = *reinterpret_cast<const uint2 *>(st + (size_t)NQ * n * 16 + t * 8);
+        w[4 * NQ] = v.x;
+        w[4 * NQ + 1] = v.y;
+    } else if constexpr (TB == 4) {
+        w[4 * NQ] = *reinterpret_cast<const uint32_t *>(st + (size_t)NQ * n * 16 + t * 4);
+    }
+}
+
 // ---------------------------------------------------------------- float-float helpers
 struct DD {
     float h, l;
@@ -180,6 +215,16 @@ __device__ __forceinline__ void dd_add(DAcc &a, const DAcc &b)
 }
 
 // ---------------------------------------------------------------- precision traits
+// F32 and F64X vectors: blocks of 32 sites, 16-byte chunk q of all 32 lanes contiguous, chunk after
+// chunk, then the 8-byte tails (as the links), so that a warp's gather of one chunk touches only the
+// cache lines it needs: of whole 24-byte records one after the other every 8-byte access touched 6
+// lines, 18 per gather instead of 6.
+// byte offset of chunk 0 of site s, records of SB bytes (the next chunk is 512 further)
+template <int SB>
+__device__ __forceinline__ size_t blocked_off(uint32_t s) { return (size_t)(s >> 5) * (32 * SB) + (s & 31) * 16; }
+// from the only chunk of a 24-byte record to its tail
+__device__ __forceinline__ int tail_step(uint32_t s) { return 512 - 8 * (int)(s & 31); }
+
 template <int P> struct Prec;
 
 // IEEE double, DFMA arithmetic
@@ -189,6 +234,13 @@ template <> struct Prec<HISQ_F64> {
     struct Vec { double v[6]; };
     struct Acc { double v[6]; };
     static constexpr int SB = 48;
+    // chunk q of site s, and the record's words as a vector
+    __device__ static size_t chunk_off(uint32_t s, int q) { return (size_t)s * SB + 16 * q; }
+    __device__ static void vec_words(const uint32_t (&w)[12], Vec &v)
+    {
+#pragma unroll
+        for (int i = 0; i < 6; i++) v.v[i] = __hiloint2double((int)w[2 * i + 1], (int)w[2 * i]);
+    }
     template <int NREAL>
     __device__ static void unpack(const uint32_t *w, Link &U)
     {
@@ -341,7 +393,11 @@ struct FloatArith {
         for (int i = 0; i < 6; i++) out.v[i] = fmaf(a, x.v[i], out.v[i]);
     }
     static constexpr bool kSplitDirections = false;
-    __device__ static void add_acc(Acc &, const Acc &) {}
+    __device__ static void add_acc(Acc &a, const Acc &b)
+    {
+#pragma unroll
+        for (int i = 0; i < 6; i++) a.v[i] += b.v[i];
+    }
     // a += the same accumulator of lane (lane ^ off)
     __device__ static void shfl_xor_add(Acc &a, int off)
     {
@@ -366,6 +422,12 @@ struct FloatArith {
 
 template <> struct Prec<HISQ_F32> : FloatArith {
     static constexpr int SB = 24;
+    __device__ static size_t chunk_off(uint32_t s, int q) { return blocked_off<SB>(s) + (q ? tail_step(s) : 0); }
+    __device__ static void vec_words(const uint32_t (&w)[6], Vec &v)
+    {
+#pragma unroll
+        for (int i = 0; i < 6; i++) v.v[i] = __uint_as_float(w[i]);
+    }
     template <int NREAL>
     __device__ static void unpack(const uint32_t *w, Link &U)
     {
@@ -374,37 +436,42 @@ template <> struct Prec<HISQ_F32> : FloatArith {
     }
     __device__ static void load(const void *base, uint32_t s, Vec &v)
     {
-        const float2 *p = reinterpret_cast<const float2 *>(static_cast<const char *>(base) + (size_t)s * SB);
-#pragma unroll
-        for (int i = 0; i < 3; i++) {
-            float2 d = __ldg(p + i);
-            v.v[2 * i] = d.x;
-            v.v[2 * i + 1] = d.y;
-        }
+        const char *p = static_cast<const char *>(base) + blocked_off<SB>(s);
+        const float4 a = __ldg(reinterpret_cast<const float4 *>(p));
+        const float2 b = __ldg(reinterpret_cast<const float2 *>(p + tail_step(s)));
+        v.v[0] = a.x; v.v[1] = a.y; v.v[2] = a.z; v.v[3] = a.w; v.v[4] = b.x; v.v[5] = b.y;
     }
     __device__ static void store(void *base, uint32_t s, const Acc &a)
     {
-        float2 *p = reinterpret_cast<float2 *>(static_cast<char *>(base) + (size_t)s * SB);
-#pragma unroll
-        for (int i = 0; i < 3; i++) p[i] = make_float2(a.v[2 * i], a.v[2 * i + 1]);
+        char *p = static_cast<char *>(base) + blocked_off<SB>(s);
+        *reinterpret_cast<float4 *>(p) = make_float4(a.v[0], a.v[1], a.v[2], a.v[3]);
+        *reinterpret_cast<float2 *>(p + tail_step(s)) = make_float2(a.v[4], a.v[5]);
     }
     // ordinary (coherent) loads, for vectors that other blocks of the same launch write
     // between grid barriers: the read-only path of load() may serve such data stale
     __device__ static void load_coh(const void *base, uint32_t s, Vec &v)
     {
-        const float2 *p = reinterpret_cast<const float2 *>(static_cast<const char *>(base) + (size_t)s * SB);
-#pragma unroll
-        for (int i = 0; i < 3; i++) {
-            const float2 d = p[i];
-            v.v[2 * i] = d.x;
-            v.v[2 * i + 1] = d.y;
-        }
+        const char *p = static_cast<const char *>(base) + blocked_off<SB>(s);
+        const float4 a = *reinterpret_cast<const float4 *>(p);
+        const float2 b = *reinterpret_cast<const float2 *>(p + tail_step(s));
+        v.v[0] = a.x; v.v[1] = a.y; v.v[2] = a.z; v.v[3] = a.w; v.v[4] = b.x; v.v[5] = b.y;
     }
 };
 
 // 16-bit storage; spinor record = 3 x (2 x 16-bit) + float scale
 template <class H2> struct Half16 : FloatArith {
     static constexpr int SB = 16;
+    __device__ static size_t chunk_off(uint32_t s, int) { return (size_t)s * SB; }
+    __device__ static void vec_words(const uint32_t (&w)[4], Vec &v)
+    {
+        const float sc = __uint_as_float(w[3]);
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            const float2 a = to2(w[i]);
+            v.v[2 * i] = a.x * sc;
+            v.v[2 * i + 1] = a.y * sc;
+        }
+    }
     __device__ static float2 to2(uint32_t w)
     {
         H2 h = *reinterpret_cast<const H2 *>(&w);
@@ -461,6 +528,15 @@ template <> struct Prec<HISQ_F64X> {
     struct Vec { float h[6], l[6]; };
     struct Acc { DAcc v[6]; };
     static constexpr int SB = 48;
+    __device__ static size_t chunk_off(uint32_t s, int q) { return blocked_off<SB>(s) + 512 * q; }
+    __device__ static void vec_words(const uint32_t (&w)[12], Vec &v)
+    {
+#pragma unroll
+        for (int i = 0; i < 6; i++) {
+            v.h[i] = __uint_as_float(w[i]);
+            v.l[i] = __uint_as_float(w[6 + i]);
+        }
+    }
     template <int NREAL>
     __device__ static void unpack(const uint32_t *w, Link &U)
     {
@@ -477,8 +553,8 @@ template <> struct Prec<HISQ_F64X> {
     }
     __device__ static void load(const void *base, uint32_t s, Vec &v)
     {
-        const float4 *p = reinterpret_cast<const float4 *>(static_cast<const char *>(base) + (size_t)s * SB);
-        float4 a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2);
+        const float4 *p = reinterpret_cast<const float4 *>(static_cast<const char *>(base) + blocked_off<SB>(s));
+        float4 a = __ldg(p), b = __ldg(p + 32), c = __ldg(p + 64);
         v.h[0] = a.x; v.h[1] = a.y; v.h[2] = a.z; v.h[3] = a.w; v.h[4] = b.x; v.h[5] = b.y;
         v.l[0] = b.z; v.l[1] = b.w; v.l[2] = c.x; v.l[3] = c.y; v.l[4] = c.z; v.l[5] = c.w;
     }
@@ -487,10 +563,10 @@ template <> struct Prec<HISQ_F64X> {
         DD d[6];
 #pragma unroll
         for (int i = 0; i < 6; i++) d[i] = dd_norm(a.v[i]);
-        float4 *p = reinterpret_cast<float4 *>(static_cast<char *>(base) + (size_t)s * SB);
+        float4 *p = reinterpret_cast<float4 *>(static_cast<char *>(base) + blocked_off<SB>(s));
         p[0] = make_float4(d[0].h, d[1].h, d[2].h, d[3].h);
-        p[1] = make_float4(d[4].h, d[5].h, d[0].l, d[1].l);
-        p[2] = make_float4(d[2].l, d[3].l, d[4].l, d[5].l);
+        p[32] = make_float4(d[4].h, d[5].h, d[0].l, d[1].l);
+        p[64] = make_float4(d[2].l, d[3].l, d[4].l, d[5].l);
     }
     __device__ static double comp(const Acc &a, int i) { return (double)a.v[i].h + (double)a.v[i].e; }
     __device__ static double vcomp(const Vec &v, int i) { return (double)v.h[i] + (double)v.l[i]; }

@@ -123,10 +123,10 @@ template <> struct Blas<HISQ_F64X> {
     }
     __device__ static void store(char *base, uint32_t s, const Vec &x)
     {
-        float4 *q = reinterpret_cast<float4 *>(base + (size_t)s * T::SB);
+        float4 *q = reinterpret_cast<float4 *>(base + blocked_off<T::SB>(s));
         q[0] = make_float4(x.h[0], x.h[1], x.h[2], x.h[3]);
-        q[1] = make_float4(x.h[4], x.h[5], x.l[0], x.l[1]);
-        q[2] = make_float4(x.l[2], x.l[3], x.l[4], x.l[5]);
+        q[32] = make_float4(x.h[4], x.h[5], x.l[0], x.l[1]);
+        q[64] = make_float4(x.l[2], x.l[3], x.l[4], x.l[5]);
     }
     __device__ static double get(const Vec &x, int i) { return (double)x.h[i] + (double)x.l[i]; }
     __device__ static void set(Vec &x, int i, double d)

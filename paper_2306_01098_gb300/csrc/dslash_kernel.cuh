@@ -112,23 +112,112 @@ __device__ __forceinline__ void vec_load(const char *base, uint32_t s, typename 
     else T::load(base, s, v);
 }
 
-// ---------------------------------------------------------------- FP64 sites in fixed point
-// hop number q2 = 2 mu + type of the site's eight pairs of hops
-struct FxHop {
-    uint32_t w[36];
-    uint32_t sn; // the neighbour the hop comes from
+// ---------------------------------------------------------------- hops through shared memory
+// The hops of a site, each thread for itself: the link and the NR vectors of a hop are copied
+// asynchronously into the thread's part of one of ST stages, ST hops before they are used, so that
+// the requests in flight cost no registers and nothing keeps a warp from running ahead.  No thread
+// reads another's part: the only waits are the thread's own (cp.async groups, one per hop).
+// Used where registers limit the warps in flight: the fixed-point FP64 sites (a hop's link is 36
+// registers; 137 -> 131 us for the 32^3 x 8 normal operator, 905 -> 853 us for a 64^3 x 16 Dslash,
+// 0.87 of the HBM rate) and FP32 vectors with four or more right-hand sides a thread (or two, with
+// the third rows of 12-real links to rebuild): 32^3 x 16, 16-bit links, 8 right-hand sides, 159 -> 142 ms
+// a solve.  With one or two right-hand sides of 18-real links the extra trip costs more than the
+// registers do (FP32 64^3 x 16 467 -> 479 us, float pairs 18 x 22 x 14 x 10, three sides, 83 -> 94 us).
+// Two stages fill the memory pipe; with four threads per site (lattices that leave the chip half
+// empty) all four hops of a thread are in flight at once.
+template <int PL, int PV, int NREAL, int NR, int DS>
+struct PipeShape {
+    static constexpr bool FX = PL == HISQ_F64 && NREAL == 18;
+    static constexpr bool on = FX || (PV != HISQ_F64 && PV != HISQ_F64X && NR >= (NREAL == 12 ? 2 : 4));
+    static constexpr int LB = NREAL == 18 ? LinkBytes<PL>::b18 : LinkBytes<PL>::b12;
+    static constexpr int VB = Prec<PV>::SB;
+    static constexpr int stage = LB + NR * VB; // bytes per thread and stage
+    static constexpr int ST = FX && NR == 1 && DS == 4 ? 4 : 2;
+    static constexpr int bytes = on ? ST * stage : 0; // per thread
 };
-template <bool BACK>
-__device__ __forceinline__ void fx_hop_issue(const DslashArgs &a, const Geom &g, const char *links, size_t slot_bytes,
-                                             const Site &c, uint32_t s, int q2, bool hint, FxHop &x)
+
+template <int PL, int PV, int NREAL, int NR, int DS, bool LL1>
+__device__ __forceinline__ void pipe_issue(const DslashArgs &a, const Geom &g, const char *links, size_t slot_bytes,
+                                           const char *in, const Site &c, uint32_t s, int mu, int h, char *st)
 {
-    const int mu = q2 >> 1, type = q2 & 1, k = type ? 3 : 1;
-    bool wrap;
-    x.sn = neighbour(g, c, s, mu, BACK ? -k : k, wrap);
-    const int lp = BACK ? 1 - a.p : a.p;
-    load_link_words<144>(links + (size_t)((lp * 2 + type) * 4 + mu) * slot_bytes, BACK ? x.sn : s, x.w, hint);
+    using P = PipeShape<PL, PV, NREAL, NR, DS>;
+    const uint32_t n = blockDim.x, t = threadIdx.x;
+    const int k = h == 0 ? 1 : h == 1 ? -1 : h == 2 ? 3 : -3, type = h >> 1;
+    const bool back = h & 1;
+    uint32_t sn;
+    if constexpr (DS > 1) {
+        sn = neighbour_any(g, c, s, mu, k);
+    } else {
+        bool wrap;
+        sn = neighbour(g, c, s, mu, k, wrap);
+    }
+    const int lp = back ? 1 - a.p : a.p;
+    const uint32_t sl = back ? sn : s, lane = sl & 31;
+    const char *blk = links + (size_t)((lp * 2 + type) * 4 + mu) * slot_bytes + (size_t)(sl >> 5) * (32 * P::LB);
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(st);
+    constexpr int NQ = P::LB / 16, TB = P::LB % 16;
+#pragma unroll
+    for (int q = 0; q < NQ; q++) cp_async<16, LL1>(dst + (q * n + t) * 16, blk + q * 512 + lane * 16);
+    if constexpr (TB > 0) cp_async<TB, true>(dst + NQ * n * 16 + t * TB, blk + NQ * 512 + lane * TB);
+    constexpr int VQ = P::VB / 16, VT = P::VB % 16;
+#pragma unroll
+    for (int r = 0; r < NR; r++) {
+        const char *v = in + (size_t)r * a.rhs_bytes;
+        const uint32_t d = dst + n * (uint32_t)(P::LB + r * P::VB);
+#pragma unroll
+        for (int q = 0; q < VQ; q++) cp_async<16, true>(d + (q * n + t) * 16, v + Prec<PV>::chunk_off(sn, q));
+        if constexpr (VT > 0) cp_async<VT, true>(d + VQ * n * 16 + t * VT, v + Prec<PV>::chunk_off(sn, VQ));
+    }
 }
 
+// the stages of one site's hops: for m = 0 .. 4/DS - 1 and h = 0 .. 3 (hops +1, -1, +3, -3 along
+// direction part 4/DS + m): link(h, w), vec(h, r, x) for every r, then next(m, h)
+template <int PL, int PV, int NREAL, int NR, int DS, bool LL1>
+struct HopPipe {
+    using P = PipeShape<PL, PV, NREAL, NR, DS>;
+    static constexpr int NMU = 4 / DS, ST = P::ST;
+    const DslashArgs &a;
+    const Geom &g;
+    const char *links;
+    size_t slot_bytes;
+    const char *in;
+    const Site &c;
+    uint32_t s;
+    int mu0;
+    char *smem;
+
+    __device__ __forceinline__ char *stage(int h) const { return smem + (size_t)(h % ST) * blockDim.x * P::stage; }
+    __device__ __forceinline__ void issue(int mu, int h)
+    {
+        pipe_issue<PL, PV, NREAL, NR, DS, LL1>(a, g, links, slot_bytes, in, c, s, mu, h, stage(h));
+    }
+    __device__ __forceinline__ void start()
+    {
+#pragma unroll
+        for (int h = 0; h < ST; h++) {
+            issue(mu0, h);
+            cp_commit();
+        }
+    }
+    __device__ __forceinline__ void link(int h, uint32_t (&w)[P::LB / 4])
+    {
+        cp_wait<ST - 1>();
+        stage_read<P::LB>(stage(h), blockDim.x, threadIdx.x, w);
+    }
+    __device__ __forceinline__ void vec(int h, int r, uint32_t (&x)[P::VB / 4])
+    {
+        stage_read<P::VB>(stage(h) + blockDim.x * (uint32_t)(P::LB + r * P::VB), blockDim.x, threadIdx.x, x);
+    }
+    // hop (m, h) has been used: its stage takes the one ST hops later
+    __device__ __forceinline__ void next(int m, int h)
+    {
+        const int mn = m + ((h + ST) >> 2);
+        if (mn < NMU) issue(mu0 + mn, (h + ST) & 3);
+        cp_commit();
+    }
+};
+
+// ---------------------------------------------------------------- FP64 sites in fixed point
 // the hops q2 in [q0, q1) of site s in FP64, one at a time: sites that hold what the fixed-point
 // format cannot (infinities, NaN, extreme magnitudes)
 static __device__ __noinline__ void fx_site_f64(const DslashArgs &a, const Geom &g, const char *links, size_t slot_bytes,
@@ -162,12 +251,8 @@ static __device__ __noinline__ void fx_site_f64(const DslashArgs &a, const Geom 
 }
 
 // D in at site s for NR right-hand sides in fixed point (fixed.cuh), the directions of one of DS
-// threads per site, summed over these threads.
-// The links of the next hop and the vector of the next product are loaded before the current one
-// is worked on: its branches (a larger exponent, a vector of zeros) would keep the compiler from
-// moving the loads there.  The hops are a loop of eight pairs, which keeps the code in the
-// instruction cache.
-template <int NR, int DS>
+// threads per site, summed over these threads
+template <int NR, int DS, bool LL1>
 __device__ __forceinline__ void fx_site(const DslashArgs &a, const Geom &g, const char *links, size_t slot_bytes,
                                         const char *in, uint32_t s, bool live, int part,
                                         Prec<HISQ_F64>::Acc (&out)[NR])
@@ -178,39 +263,33 @@ __device__ __forceinline__ void fx_site(const DslashArgs &a, const Geom &g, cons
 #pragma unroll
     for (int r = 0; r < NR; r++) fx_zero(acc[r]);
     if (live) {
-        const bool hint = NR > 1 && a.stream_links != 0;
+        extern __shared__ __align__(16) char pipe_smem[];
         const Site c = site_coords(g, s, a.p);
-        FxHop fw, bw;
-        FxVec v[2]; // product number parity: the current one and the next
-        fx_hop_issue<false>(a, g, links, slot_bytes, c, s, q0, hint, fw);
-        fx_load(in, fw.sn, v[0]);
+        HopPipe<HISQ_F64, HISQ_F64, 18, NR, DS, LL1> pipe{a, g, links, slot_bytes, in, c, s, part * (4 / DS), pipe_smem};
+        pipe.start();
 #pragma unroll 1
-        for (int q2 = q0; q2 < q0 + NQ; q2++) {
-            fx_hop_issue<true>(a, g, links, slot_bytes, c, s, q2, hint, bw);
-            uint32_t code = fx_code(fw.w);
+        for (int m = 0; m < 4 / DS; m++)
 #pragma unroll
-            for (int r = 0; r < NR; r++) {
-                fx_load(in + (r + 1 < NR ? (size_t)(r + 1) * a.rhs_bytes : 0), r + 1 < NR ? fw.sn : bw.sn, v[(r + 1) & 1]);
-                fx_hop<false>(acc[r], fw.w, code, v[r & 1]);
-            }
-            const int qn = q2 + 1 < q0 + NQ ? q2 + 1 : q0; // (the last one is not used)
-            fx_hop_issue<false>(a, g, links, slot_bytes, c, s, qn, hint, fw);
-            code = fx_code(bw.w);
+            for (int h = 0; h < 4; h++) {
+                uint32_t w[36];
+                pipe.link(h, w);
+                const uint32_t code = fx_code(w);
 #pragma unroll
-            for (int r = 0; r < NR; r++) {
-                fx_load(in + (r + 1 < NR ? (size_t)(r + 1) * a.rhs_bytes : 0), r + 1 < NR ? bw.sn : fw.sn,
-                        v[(NR + r + 1) & 1]);
-                fx_hop<true>(acc[r], bw.w, code, v[(NR + r) & 1]);
+                for (int r = 0; r < NR; r++) {
+                    uint32_t x[12];
+                    pipe.vec(h, r, x);
+                    if (h & 1) fx_hop<true>(acc[r], w, code, x);
+                    else fx_hop<false>(acc[r], w, code, x);
+                }
+                pipe.next(m, h);
             }
-        }
     }
     bool bad = false;
 #pragma unroll
     for (int r = 0; r < NR; r++) {
         if constexpr (DS > 1) fx_combine<DS>(acc[r]);
-        const double sc = fx_scale(acc[r]);
 #pragma unroll
-        for (int k = 0; k < 6; k++) out[r].v[k] = fx_value(acc[r], k, sc);
+        for (int k = 0; k < 6; k++) out[r].v[k] = fx_value(acc[r], k);
         bad |= acc[r].bad;
     }
     if (__any_sync(0xffffffffu, bad)) {
@@ -222,7 +301,7 @@ __device__ __forceinline__ void fx_site(const DslashArgs &a, const Geom &g, cons
 #pragma unroll
             for (int k = 0; k < 6; k++) {
 #pragma unroll
-                for (int off = DS / 2; off > 0; off >>= 1) o[k] += __shfl_xor_sync(0xffffffffu, o[k], off);
+                for (int off = 16; off >= 32 / DS; off >>= 1) o[k] += __shfl_xor_sync(0xffffffffu, o[k], off);
                 if (acc[r].bad) out[r].v[k] = o[k];
             }
         }
@@ -242,8 +321,9 @@ __device__ __forceinline__ void fx_site(const DslashArgs &a, const Geom &g, cons
 // are the same addresses in the same instruction (one request), so a link is fetched once
 // for all NR RG right-hand sides with 1/RG of the accumulators per thread.
 // LL1: links allocate in L1 (right-hand-side groups of one block read the same links).
+// PIPE: the hops' operands come through shared memory (pipe_hops); else through registers.
 template <int PL, int PV, int NREAL, int NR, int EPI, int DS, bool COH = false, bool PF = false, int RG = 1,
-          class DT = double, bool LL1 = false>
+          class DT = double, bool LL1 = false, bool PIPE = false>
 __device__ __forceinline__ void dslash_item(const DslashArgs &a, const Geom &g, const char *links, size_t slot_bytes,
                                             std::conditional_t<std::is_same<DT, FF>::value, float, double> sc0,
                                             std::conditional_t<std::is_same<DT, FF>::value, float, double> sc1,
@@ -263,11 +343,18 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const Geom &g, 
     using TL = Prec<PL>; // link storage
     constexpr int LB = NREAL == 18 ? LinkBytes<PL>::b18 : LinkBytes<PL>::b12;
     constexpr bool TWO = (PL == HISQ_F16 || PL == HISQ_BF16 || NREAL == 12);
-    constexpr bool SPLIT = T::kSplitDirections;
+    // directions summed apart: always for float pairs; for FP32 with one right-hand side, so that a
+    // site's error does not depend on how many threads share it (measured 1.9e-7 with one running sum,
+    // 1.2e-7 apart; the gathers hide the 24 additions)
+    constexpr bool SPLIT = T::kSplitDirections || (PL == HISQ_F32 && NR == 1 && !TWO && !COH && DS < 4);
     constexpr int NMU = 4 / DS;
     const uint32_t gt = tile * (uint32_t)a.bs + tid;
-    const uint32_t u = gt / (DS * RG); // site number in launch order
-    const int part = (int)(gt % DS);
+    // site number in launch order, and this thread's directions: with DS > 1 a warp holds 32 / DS
+    // sites, lanes in groups of 32 / DS per part, so that a quarter-warp's 16-byte accesses still fall
+    // into one line (lanes of one site side by side spread them over DS)
+    constexpr uint32_t kSites = 32 / DS;
+    const uint32_t u = DS > 1 ? (gt >> 5) * kSites + (gt & (kSites - 1)) : gt / RG;
+    const int part = DS > 1 ? (int)((gt & 31) / kSites) : 0;
     if constexpr (RG > 1) {
         const size_t goff = (size_t)(gt % RG) * NR * a.rhs_bytes;
         in += goff;
@@ -289,7 +376,8 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const Geom &g, 
 
     // FP64 with 18 reals: in fixed point, summed over the site's threads there
     constexpr bool FX = PL == HISQ_F64 && NREAL == 18;
-    if constexpr (FX) fx_site<NR, DS>(a, g, links, slot_bytes, in, s, live, part, out);
+    static_assert(!FX || PIPE, "the fixed-point sites read their operands from shared memory");
+    if constexpr (FX) fx_site<NR, DS, LL1>(a, g, links, slot_bytes, in, s, live, part, out);
     else if (live) {
         const Site c = site_coords(g, s, a.p);
         typename T::Acc acc[TWO ? 2 : 1][NR];
@@ -298,6 +386,47 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const Geom &g, 
 #pragma unroll
             for (int r = 0; r < NR; r++) T::zero(acc[t][r]);
 
+        if constexpr (PIPE) {
+            extern __shared__ __align__(16) char pipe_smem[];
+            HopPipe<PL, PV, NREAL, NR, DS, LL1> pipe{a, g, links, slot_bytes, in, c, s, part * NMU, pipe_smem};
+            pipe.start();
+#pragma unroll 1
+            for (int m = 0; m < NMU; m++) {
+                typename T::Acc dacc[SPLIT ? NR : 1];
+                if constexpr (SPLIT) {
+#pragma unroll
+                    for (int r = 0; r < NR; r++) T::zero(dacc[r]);
+                }
+#pragma unroll
+                for (int h = 0; h < 4; h++) {
+                    uint32_t w[LB / 4];
+                    pipe.link(h, w);
+                    typename T::Link U;
+                    TL::template unpack<NREAL>(w, U);
+                    if constexpr (NREAL == 12) {
+                        const int mu = part * NMU + m;
+                        bool wrap;
+                        neighbour(g, c, s, mu, h == 0 ? 1 : h == 1 ? -1 : h == 2 ? 3 : -3, wrap);
+                        T::rebuild(U, (eta_neg(c, mu) != 0) ^ (mu == 3 && wrap));
+                    }
+#pragma unroll
+                    for (int r = 0; r < NR; r++) {
+                        uint32_t x[T::SB / 4];
+                        pipe.vec(h, r, x);
+                        typename T::Vec v;
+                        T::vec_words(x, v);
+                        typename T::Acc &dst = SPLIT ? dacc[SPLIT ? r : 0] : acc[TWO ? h >> 1 : 0][r];
+                        if (h & 1) T::template hop<true, true>(dst, U, v);
+                        else T::template hop<false, false>(dst, U, v);
+                    }
+                    pipe.next(m, h);
+                }
+                if constexpr (SPLIT) {
+#pragma unroll
+                    for (int r = 0; r < NR; r++) T::add_acc(acc[0][r], dacc[r]);
+                }
+            }
+        } else {
 #pragma unroll
         for (int m = 0; m < NMU; m++) {
             const int mu = part * NMU + m;
@@ -371,6 +500,7 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const Geom &g, 
                 }
             }
         }
+        }
 #pragma unroll
         for (int r = 0; r < NR; r++) {
             if constexpr (TWO) {
@@ -384,7 +514,7 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const Geom &g, 
     // partial sums of the DS threads of a site meet in every one of them
     if constexpr (DS > 1 && !FX) {
 #pragma unroll
-        for (int off = DS / 2; off > 0; off >>= 1)
+        for (int off = 16; off >= (int)kSites; off >>= 1)
 #pragma unroll
             for (int r = 0; r < NR; r++) T::shfl_xor_add(out[r], off);
     }
@@ -436,8 +566,18 @@ __device__ __forceinline__ double dot_value(double x) { return x; }
 // a.bs threads over the same sites, slice g taking the g-th of the block's WG groups of NR
 // right-hand sides; their link loads allocate in L1, so one L2 read of a link serves the
 // block's WG NR right-hand sides without the registers of WG NR accumulators per thread.
+// 256-thread blocks per SM that the registers are limited for.  Left alone the compiler moves the
+// loads of all 16 hops to the front of the site (250 registers, 8 warps an SM); the gathers want warps:
+// FP32 vectors 48 / 64 / 128 registers at 1 / 2 / 4 right-hand sides a thread (14-shift FP32 solve
+// 32^3 x 8: 74 ms without limits, 63 ms with 64 / 80 / 128, 59 ms so), FP64 and float pairs 128 at one.
+constexpr int min_blocks(int pl, int pv, int nreal, int nr)
+{
+    if (pv == HISQ_F64 || pv == HISQ_F64X) return nr == 1 && !(pl == HISQ_F64 && nreal == 12) ? 2 : 1;
+    const int less = nreal == 12 ? 1 : 0; // (the rebuilt third row)
+    return nr == 1 ? 5 - less : nr == 2 ? 4 - less : nr == 4 ? 2 : 1;
+}
 template <int PL, int PV, int NREAL, int NR, int EPI, int DS, bool BATCH, int RG = 1, int WG = 1>
-__global__ void __launch_bounds__(kDslashMaxBlock) k_dslash(const DslashArgs a)
+__global__ void __launch_bounds__(kDslashMaxBlock, min_blocks(PL, PV, NREAL, NR)) k_dslash(const DslashArgs a)
 {
     static_assert(WG == 1 || (EPI == 0 && DS == 1 && RG == 1 && !BATCH), "block slices: plain Dslash, one thread per site");
     using T = Prec<PV>;
@@ -492,7 +632,7 @@ __global__ void __launch_bounds__(kDslashMaxBlock) k_dslash(const DslashArgs a)
             DTK td[ND];
 #pragma unroll
             for (int j = 0; j < ND; j++) td[j] = DTK{};
-            dslash_item<PL, PV, NREAL, 1, EPI, DS, false, false, 1, DTK>(
+            dslash_item<PL, PV, NREAL, 1, EPI, DS, false, false, 1, DTK, false, PipeShape<PL, PV, NREAL, 1, DS>::on>(
                 a, sg, L.links[PL], L.slot_bytes[PL], sc0, sc1, a.in + off, a.out + off, EPI ? a.pv + off : nullptr,
                 EPI == 2 ? a.rv + off : nullptr, a.shift ? a.shift + k : nullptr, tile, td);
             if constexpr (EPI >= 1) {
@@ -528,7 +668,7 @@ __global__ void __launch_bounds__(kDslashMaxBlock) k_dslash(const DslashArgs a)
         const auto sc0 = [&] { if constexpr (FFK) return a.scale_f[0]; else return a.scale[0]; }();
         const auto sc1 = [&] { if constexpr (FFK) return a.scale_f[1]; else return a.scale[1]; }();
         for (uint32_t item = blockIdx.x; item < a.items; item += gridDim.x)
-            dslash_item<PL, PV, NREAL, NR, EPI, DS, false, false, RG, DTK, (WG > 1)>(
+            dslash_item<PL, PV, NREAL, NR, EPI, DS, false, false, RG, DTK, (WG > 1), PipeShape<PL, PV, NREAL, NR, DS>::on>(
                 a, a.g, a.links, a.slot_bytes, sc0, sc1, a.in + off, a.out + off, EPI ? a.pv + off : nullptr,
                 EPI == 2 ? a.rv + off : nullptr, a.shift ? a.shift + rhs0 : nullptr, item / ngroups, dots, tid);
         if constexpr (EPI >= 1) {
@@ -562,12 +702,18 @@ static cudaError_t launch_one(const DslashArgs &a0, cudaStream_t st)
     const int bs = BATCH ? kDslashBlock : a.bs;
     if (bs != 64 && bs != 128 && bs != 256) return cudaErrorInvalidValue;
     a.bs = bs;
+    const size_t smem = (size_t)bs * PipeShape<PL, PV, NREAL, NR, DS>::bytes;
+    if (smem > 32 * 1024) { // (48 KB with the static part) a per-device attribute of the function
+        cudaError_t e = cudaFuncSetAttribute(k_dslash<PL, PV, NREAL, NR, EPI, DS, BATCH, RG, WG>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
     static int occ[3] = {-1, -1, -1}; // resident blocks per SM of this instantiation, per block size
     const int bi = bs == 64 ? 0 : bs == 128 ? 1 : 2;
     if (occ[bi] < 0) {
         int o = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_dslash<PL, PV, NREAL, NR, EPI, DS, BATCH, RG, WG>, bs,
-                                                          0) != cudaSuccess ||
+                                                          smem) != cudaSuccess ||
             o < 1)
             o = 1;
         occ[bi] = o;
@@ -580,7 +726,7 @@ static cudaError_t launch_one(const DslashArgs &a0, cudaStream_t st)
         a.items = items;
         a.red.nblocks = (int)a.batch_maxtiles[d]; // partials per lattice (zero beyond its tiles)
         a.red.ntotal = (int)blocks;
-        k_dslash<PL, PV, NREAL, 1, EPI, DS, true><<<blocks, kDslashBlock, 0, st>>>(a);
+        k_dslash<PL, PV, NREAL, 1, EPI, DS, true><<<blocks, kDslashBlock, smem, st>>>(a);
         return cudaGetLastError();
     } else {
         const int ts = bs / WG; // threads over the sites of one tile (one slice of the block)
@@ -595,7 +741,7 @@ static cudaError_t launch_one(const DslashArgs &a0, cudaStream_t st)
         a.items = (uint32_t)items;
         a.red.nblocks = (int)(blocks / ng); // partials per right-hand side
         a.red.ntotal = (int)blocks;
-        k_dslash<PL, PV, NREAL, NR, EPI, DS, false, RG, WG><<<(unsigned)blocks, bs, 0, st>>>(a);
+        k_dslash<PL, PV, NREAL, NR, EPI, DS, false, RG, WG><<<(unsigned)blocks, bs, smem, st>>>(a);
         return cudaGetLastError();
     }
 }

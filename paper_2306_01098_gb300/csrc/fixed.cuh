@@ -34,7 +34,8 @@ namespace hisq {
 constexpr uint32_t kFxRaw = 0xfff;
 constexpr uint32_t kFxMinExp = 64; // smallest biased exponent of a link or vector in fixed point
 // biased exponents of products (sum of two biased exponents) that the sums are formed with
-constexpr uint32_t kFxELo = 1100, kFxEHi = 3000;
+// (results, whose last bit is 2^-85 of the largest product, stay normal numbers)
+constexpr uint32_t kFxELo = 1200, kFxEHi = 3000;
 
 __host__ __device__ inline void fx_encode_link(const double (&d)[18], uint32_t (&w)[36])
 {
@@ -135,37 +136,20 @@ __device__ __forceinline__ void fx_fold(FxAcc &a)
     }
 }
 
-// one colour vector as its doubles' words (lo, hi)
-struct FxVec {
-    uint32_t lo[6], hi[6];
-};
-
-__device__ __forceinline__ void fx_load(const char *base, uint32_t s, FxVec &v)
-{
-    const uint4 *p = reinterpret_cast<const uint4 *>(base + (size_t)s * 48);
-#pragma unroll
-    for (int i = 0; i < 3; i++) {
-        const uint4 q = __ldg(p + i);
-        v.lo[2 * i] = q.x;
-        v.hi[2 * i] = q.y;
-        v.lo[2 * i + 1] = q.z;
-        v.hi[2 * i + 1] = q.w;
-    }
-}
-
-// a += U v (BACK = false) or a -= U^+ v (BACK = true); w: the stored link, code: its exponent
+// a += U v (BACK = false) or a -= U^+ v (BACK = true); w: the stored link, code: its exponent,
+// v: the words of the vector's six doubles
 template <bool BACK>
-__device__ __forceinline__ void fx_hop(FxAcc &a, const uint32_t (&w)[36], uint32_t code, const FxVec &v)
+__device__ __forceinline__ void fx_hop(FxAcc &a, const uint32_t (&w)[36], uint32_t code, const uint32_t (&v)[12])
 {
     uint32_t top = 0;
 #pragma unroll
-    for (int k = 0; k < 6; k++) top = max(top, v.hi[k] & 0x7fffffffu);
+    for (int k = 0; k < 6; k++) top = max(top, v[2 * k + 1] & 0x7fffffffu);
     const uint32_t ev = top >> 20, e = code ? code + ev : 0u;
     if (ev - kFxMinExp >= 0x7ffu - kFxMinExp || e - kFxELo > kFxEHi - kFxELo) {
         // zeros contribute nothing; anything else here is left to FP64
         uint32_t any = 0;
 #pragma unroll
-        for (int k = 0; k < 6; k++) any |= (v.hi[k] & 0x7fffffffu) | v.lo[k];
+        for (int k = 0; k < 6; k++) any |= (v[2 * k + 1] & 0x7fffffffu) | v[2 * k];
         a.bad |= any != 0 && (code != 0 || ev == 0x7ffu);
         return;
     }
@@ -177,11 +161,11 @@ __device__ __forceinline__ void fx_hop(FxAcc &a, const uint32_t (&w)[36], uint32
     int32_t h[6], l[6], nh[3], nl[3];
 #pragma unroll
     for (int k = 0; k < 6; k++) {
-        const uint32_t s = t - ((v.hi[k] >> 20) & 0x7ffu);
-        const uint32_t mh = (v.hi[k] & 0xfffffu) | 0x100000u;
-        uint64_t m = (uint64_t)__funnelshift_l(v.lo[k], mh, 7) << 32 | (v.lo[k] << 7);
+        const uint32_t s = t - ((v[2 * k + 1] >> 20) & 0x7ffu);
+        const uint32_t mh = (v[2 * k + 1] & 0xfffffu) | 0x100000u;
+        uint64_t m = (uint64_t)__funnelshift_l(v[2 * k], mh, 7) << 32 | (v[2 * k] << 7);
         m = s < 64 ? m >> s : 0ull;
-        const uint32_t sg = (uint32_t)((int32_t)(BACK ? ~v.hi[k] : v.hi[k]) >> 31);
+        const uint32_t sg = (uint32_t)((int32_t)(BACK ? ~v[2 * k + 1] : v[2 * k + 1]) >> 31);
         const int64_t x = (int64_t)(m ^ ((uint64_t)sg << 32 | sg)) - (int64_t)(int32_t)sg;
         l[k] = (int32_t)(uint32_t)x;
         h[k] = (int32_t)(x >> 32) + (int32_t)((uint32_t)l[k] >> 31);
@@ -223,12 +207,12 @@ __device__ __forceinline__ void fx_hop(FxAcc &a, const uint32_t (&w)[36], uint32
     fx_fold(a);
 }
 
-// sum over the DS lanes that share a site, in every one of them
+// sum over the DS lanes that share a site (32 / DS apart), in every one of them
 template <int DS>
 __device__ __forceinline__ void fx_combine(FxAcc &a)
 {
 #pragma unroll
-    for (int off = DS / 2; off > 0; off >>= 1) {
+    for (int off = 16; off >= 32 / DS; off >>= 1) {
         const uint32_t eo = __shfl_xor_sync(0xffffffffu, a.E, off);
         a.bad |= __shfl_xor_sync(0xffffffffu, (int)a.bad, off) != 0;
         if (eo > a.E) {
@@ -244,18 +228,34 @@ __device__ __forceinline__ void fx_combine(FxAcc &a)
     }
 }
 
-// component k as a double.  The three words become doubles by the exponent trick (2^52 + x and
-// the like are exact), so this takes four FP64 operations and no conversion.
-__device__ __forceinline__ double fx_value(const FxAcc &a, int k, double scale)
+// component k as a double, to nearest, on integers: FP64 operations (four per component with exact
+// splittings of the words) took 13 % of the normal operator's time at 2 a clock and SM
+__device__ __forceinline__ double fx_value(const FxAcc &a, int k)
 {
-    const uint32_t f = (uint32_t)a.M[k], lo = (uint32_t)(uint64_t)a.H[k], hi = (uint32_t)((uint64_t)a.H[k] >> 32);
-    const double xh = __hiloint2double(0x45300000, (int)(hi ^ 0x80000000u)); // 2^84 + (hi + 2^31) 2^32
-    const double xl = __hiloint2double(0x43300000, (int)lo);                 // 2^52 + lo
-    const double xf = __hiloint2double(0x41300000, (int)f);                  // 2^20 + f 2^-32
-    // 2^84 + 2^63 + 2^52
-    const double s = __dadd_rn(__dsub_rn(xh, __hiloint2double(0x45300000, (int)0x80100000u)), xl);
-    return __dmul_rn(__dadd_rn(s, __dsub_rn(xf, 1048576.0)), scale);
+    // magnitude of the 96-bit sum H 2^32 + M as words x2 x1 x0
+    const uint32_t sg = (uint32_t)((int32_t)(a.H[k] >> 32) >> 31);
+    uint32_t x0 = (uint32_t)a.M[k] ^ sg;
+    uint64_t xh = (uint64_t)a.H[k] ^ ((uint64_t)sg << 32 | sg);
+    xh += (uint64_t)(sg & (uint32_t)(x0 == 0xffffffffu)); // + 1, carried
+    x0 -= sg;
+    uint32_t x2 = (uint32_t)(xh >> 32), x1 = (uint32_t)xh;
+    int top = 95;
+#pragma unroll
+    for (int i = 0; i < 2; i++) {
+        const bool z = x2 == 0;
+        x2 = z ? x1 : x2;
+        x1 = z ? x0 : x1;
+        x0 = z ? 0u : x0;
+        top -= z ? 32 : 0;
+    }
+    const int lz = __clz((int)x2);
+    const uint32_t m1 = __funnelshift_l(x1, x2, lz), m0 = __funnelshift_l(x0, x1, lz); // leading bit on top
+    // (the leading bit adds one to the exponent field, a carry of the rounding another)
+    const int e = (int)a.E + top - lz - 2132 + 1023 - 1;
+    uint64_t m = (uint64_t)(m1 >> 11) << 32 | __funnelshift_r(m0, m1, 11);
+    m += (m0 >> 10) & 1u;
+    m += (uint64_t)((uint32_t)e << 20 | (sg & 0x80000000u)) << 32;
+    return x2 ? __longlong_as_double((long long)m) : 0.0;
 }
-__device__ __forceinline__ double fx_scale(const FxAcc &a) { return __hiloint2double((int)((a.E - 2100u + 1023u) << 20), 0); }
 
 }  // namespace hisq

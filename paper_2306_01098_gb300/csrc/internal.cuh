@@ -9,11 +9,12 @@
 //   by the lane-contiguous tail (4 or 8 bytes per lane) when the link size is not a
 //   multiple of 16.  A warp reading one chunk of 32 consecutive sites therefore reads
 //   512 contiguous bytes.
-//   Spinors (internal fields): site-major, one record per half-lattice site:
-//     F64  : 6 doubles (re, im of 3 colours)                48 B
-//     F64X : 6 hi floats then 6 lo floats                    48 B
-//     F32  : 6 floats                                        24 B
-//     F16/BF16 : 6 halves + one float scale                  16 B
+//   Spinors (internal fields), one record per half-lattice site:
+//     F64  : 6 doubles (re, im of 3 colours)                48 B   site after site
+//     F64X : 6 hi floats then 6 lo floats                    48 B   blocks of 32 sites
+//     F32  : 6 floats                                        24 B   blocks of 32 sites
+//     F16/BF16 : 6 halves + one float scale                  16 B   site after site
+//   (blocks of 32 sites: chunk q of every lane contiguous, then the tails, as the links)
 //   Multi-RHS fields are [nrhs][VhPad] records.
 #pragma once
 
@@ -116,6 +117,20 @@ __device__ __forceinline__ uint32_t neighbour(const Geom &g, const Site &c, uint
         v -= (v >= n) ? n : 0;
         return s + (v - c.t) * (int)g.st;
     }
+}
+
+// the same without branches, for a direction that differs between the lanes of a warp (a switch would
+// run the loads behind it once for every direction)
+__device__ __forceinline__ uint32_t neighbour_any(const Geom &g, const Site &c, uint32_t s, int mu, int k)
+{
+    const int x = mu == 0 ? c.x : mu == 1 ? c.y : mu == 2 ? c.z : c.t;
+    const int n = mu == 0 ? g.n[0] : mu == 1 ? g.n[1] : mu == 2 ? g.n[2] : g.n[3];
+    const int st = mu == 1 ? (int)g.sy : mu == 2 ? (int)g.sz : (int)g.st;
+    int v = x + k;
+    v += v < 0 ? n : 0;
+    v -= v >= n ? n : 0;
+    const uint32_t xs = c.row + (uint32_t)(v >> 1), os = s + (uint32_t)((v - x) * st);
+    return mu == 0 ? xs : os;
 }
 
 // MILC staggered phase eta_mu(x) as a sign bit (1 = negative)
