@@ -214,6 +214,15 @@ __device__ __forceinline__ void dd_add(DAcc &a, const DAcc &b)
     a.e = __fsub_rn(t, __fsub_rn(hi, s));
 }
 
+// exact FP32 -> FP64 on the bits: the conversion instruction issues like the FP64 unit
+__device__ __forceinline__ double widen(float x)
+{
+    const uint32_t u = __float_as_uint(x), m = u & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f800000u - 0x00800000u || m == 0) // normal or zero
+        return __hiloint2double((int)((u & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), (int)(u << 29));
+    return (double)x;
+}
+
 // ---------------------------------------------------------------- precision traits
 // F32 and F64X vectors: blocks of 32 sites, 16-byte chunk q of all 32 lanes contiguous, chunk after
 // chunk, then the 8-byte tails (as the links), so that a warp's gather of one chunk touches only the
@@ -270,6 +279,7 @@ template <> struct Prec<HISQ_F64> {
     }
     // components as doubles (for epilogues / reductions)
     __device__ static double comp(const Acc &a, int i) { return a.v[i]; }
+    __device__ static double canon(const Acc &a, int i) { return a.v[i]; }
     __device__ static double vcomp(const Vec &v, int i) { return v.v[i]; }
     __device__ static void set_acc(Acc &a, int i, double x) { a.v[i] = x; }
     __device__ static void negate(Vec &v)
@@ -350,6 +360,7 @@ struct FloatArith {
         for (int i = 0; i < 6; i++) a.v[i] = 0.f;
     }
     __device__ static double comp(const Acc &a, int i) { return (double)a.v[i]; }
+    __device__ static double canon(const Acc &a, int i) { return widen(a.v[i]); }
     __device__ static double vcomp(const Vec &v, int i) { return (double)v.v[i]; }
     __device__ static void set_acc(Acc &a, int i, double x) { a.v[i] = (float)x; }
     __device__ static void negate(Vec &v)
@@ -569,6 +580,12 @@ template <> struct Prec<HISQ_F64X> {
         p[64] = make_float4(d[2].l, d[3].l, d[4].l, d[5].l);
     }
     __device__ static double comp(const Acc &a, int i) { return (double)a.v[i].h + (double)a.v[i].e; }
+    // a component as the stored record would give it back
+    __device__ static double canon(const Acc &a, int i)
+    {
+        const DD d = dd_norm(a.v[i]);
+        return (double)d.h + (double)d.l;
+    }
     __device__ static double vcomp(const Vec &v, int i) { return (double)v.h[i] + (double)v.l[i]; }
     __device__ static void set_acc(Acc &a, int i, double x)
     {

@@ -28,7 +28,7 @@
 namespace hisq {
 
 int apply_mdagm(hisq_ctx *ctx, int prec, double m, const void *in, void *tmp, void *out, int nrhs, size_t rhs_bytes,
-                cudaStream_t st, const Reduce *red, bool tune);
+                cudaStream_t st, const Reduce *red, bool tune, double *out64 = nullptr);
 
 // ---------------------------------------------------------------- scalar bookkeeping
 enum { SC_INIT_BB = 0, SC_INIT_R = 1, SC_RU = 2 };

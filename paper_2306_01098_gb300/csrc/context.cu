@@ -207,18 +207,10 @@ __global__ void k_link_stats(const double *fat, const double *lng, size_t nlinks
 // memory: the canonical side moves as consecutive 8-byte words of consecutive threads (it is only
 // 8-byte aligned), the internal side as whole chunks.  Both are passes over memory; a thread storing
 // its own 48-byte record word by word left every warp store 32 half-filled sectors, and the exact
-// FP32 -> FP64 widening issues like the FP64 unit, so it is done on the bits.
+// FP32 -> FP64 widening issues like the FP64 unit, so it is done on the bits (widen).
 // 48^3 x 12, FP32, 8 vectors: a whole FP32 call 481 -> 418 us, the export 127 us of it before (56 us
 // at the HBM rate).
 constexpr int kFieldBlock = 256;
-
-__device__ __forceinline__ double widen(float x)
-{
-    const uint32_t u = __float_as_uint(x), m = u & 0x7fffffffu;
-    if (m - 0x00800000u < 0x7f800000u - 0x00800000u || m == 0) // normal or zero
-        return __hiloint2double((int)((u & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), (int)(u << 29));
-    return (double)x;
-}
 
 // component i of a record as a double
 template <int P>

@@ -103,6 +103,9 @@ __device__ __forceinline__ double acc_norm2(const typename T::Acc &o)
     }
 }
 
+// bytes between the right-hand sides of the output
+__device__ __forceinline__ size_t out_stride(const DslashArgs &a) { return a.out64 ? (size_t)a.g.Vh * 48 : a.rhs_bytes; }
+
 // vector load: the read-only path, or (COH) ordinary loads for vectors that other blocks of
 // the same launch write between grid barriers
 template <class T, bool COH>
@@ -358,7 +361,7 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const Geom &g, 
     if constexpr (RG > 1) {
         const size_t goff = (size_t)(gt % RG) * NR * a.rhs_bytes;
         in += goff;
-        outp += goff;
+        outp += COH ? goff : (size_t)(gt % RG) * NR * out_stride(a);
         if (pvp) pvp += goff;
         if (rvp) rvp += goff;
         if (m4r) m4r += (gt % RG) * NR;
@@ -545,7 +548,13 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const Geom &g, 
                     }
                 }
             }
-            T::store(outp + (size_t)r * a.rhs_bytes, EPI >= 1 ? s - ebase : s, out[r]);
+            if (!COH && a.out64) { // the caller's FP64 buffer, without a pass of its own
+                double2 *q = reinterpret_cast<double2 *>(outp + (size_t)r * out_stride(a) + (size_t)s * 48);
+#pragma unroll
+                for (int i = 0; i < 3; i++) q[i] = make_double2(T::canon(out[r], 2 * i), T::canon(out[r], 2 * i + 1));
+            } else {
+                T::store(outp + (size_t)r * a.rhs_bytes, EPI >= 1 ? s - ebase : s, out[r]);
+            }
         }
     }
 }
@@ -669,7 +678,7 @@ __global__ void __launch_bounds__(kDslashMaxBlock, min_blocks(PL, PV, NREAL, NR)
         const auto sc1 = [&] { if constexpr (FFK) return a.scale_f[1]; else return a.scale[1]; }();
         for (uint32_t item = blockIdx.x; item < a.items; item += gridDim.x)
             dslash_item<PL, PV, NREAL, NR, EPI, DS, false, false, RG, DTK, (WG > 1), PipeShape<PL, PV, NREAL, NR, DS>::on>(
-                a, a.g, a.links, a.slot_bytes, sc0, sc1, a.in + off, a.out + off, EPI ? a.pv + off : nullptr,
+                a, a.g, a.links, a.slot_bytes, sc0, sc1, a.in + off, a.out + (size_t)rhs0 * out_stride(a), EPI ? a.pv + off : nullptr,
                 EPI == 2 ? a.rv + off : nullptr, a.shift ? a.shift + rhs0 : nullptr, item / ngroups, dots, tid);
         if constexpr (EPI >= 1) {
             if (a.red.partials) { // uniform over the grid

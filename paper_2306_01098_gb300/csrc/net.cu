@@ -29,7 +29,7 @@
 namespace hisq {
 
 int apply_mdagm(hisq_ctx *ctx, int prec, double m, const void *in, void *tmp, void *out, int nrhs, size_t rhs_bytes,
-                cudaStream_t st, const Reduce *red, bool tune);
+                cudaStream_t st, const Reduce *red, bool tune, double *out64 = nullptr);
 
 // ---------------------------------------------------------------- activation access
 __device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }

@@ -17,7 +17,7 @@
 namespace hisq {
 
 int apply_mdagm(hisq_ctx *ctx, int prec, double m, const void *in, void *tmp, void *out, int nrhs, size_t rhs_bytes,
-                cudaStream_t st, const Reduce *red, bool tune);
+                cudaStream_t st, const Reduce *red, bool tune, double *out64 = nullptr);
 
 constexpr size_t kNoAllocScratchSites = size_t(1) << 20; // nrhs * Vh must not exceed this
 constexpr int kNoAllocMaxDevices = 64;
