@@ -136,6 +136,26 @@ __device__ __forceinline__ void fx_fold(FxAcc &a)
     }
 }
 
+// limbs of the double hi:lo for the biased exponent t (>= its own), negated if flip = ~0
+__device__ __forceinline__ void fx_limbs(uint32_t lo, uint32_t hi, uint32_t t, uint32_t flip, int32_t &h, int32_t &l)
+{
+    const uint32_t s = t - ((hi >> 20) & 0x7ffu);
+    const uint32_t mh = (hi & 0xfffffu) | 0x100000u;
+    uint64_t m = (uint64_t)__funnelshift_l(lo, mh, 7) << 32 | (lo << 7);
+    m = s < 64 ? m >> s : 0ull;
+    const uint32_t sg = (uint32_t)((int32_t)(hi ^ flip) >> 31);
+    const int64_t x = (int64_t)(m ^ ((uint64_t)sg << 32 | sg)) - (int64_t)(int32_t)sg;
+    l = (int32_t)(uint32_t)x;
+    h = (int32_t)(x >> 32) + (int32_t)((uint32_t)l >> 31);
+}
+
+// the limbs of the negative (-2^31 has none in 32 bits: its limb becomes 2^31 - 1, one unit of 2^-60 off)
+__device__ __forceinline__ void fx_neg(int32_t h, int32_t l, int32_t &nh, int32_t &nl)
+{
+    nh = -h;
+    nl = -max(-2147483647, l);
+}
+
 // a += U v (BACK = false) or a -= U^+ v (BACK = true); w: the stored link, code: its exponent,
 // v: the words of the vector's six doubles
 template <bool BACK>
@@ -160,24 +180,10 @@ __device__ __forceinline__ void fx_hop(FxAcc &a, const uint32_t (&w)[36], uint32
     const uint32_t t = a.E - code; // the vector's exponent in these sums, >= ev
     int32_t h[6], l[6], nh[3], nl[3];
 #pragma unroll
-    for (int k = 0; k < 6; k++) {
-        const uint32_t s = t - ((v[2 * k + 1] >> 20) & 0x7ffu);
-        const uint32_t mh = (v[2 * k + 1] & 0xfffffu) | 0x100000u;
-        uint64_t m = (uint64_t)__funnelshift_l(v[2 * k], mh, 7) << 32 | (v[2 * k] << 7);
-        m = s < 64 ? m >> s : 0ull;
-        const uint32_t sg = (uint32_t)((int32_t)(BACK ? ~v[2 * k + 1] : v[2 * k + 1]) >> 31);
-        const int64_t x = (int64_t)(m ^ ((uint64_t)sg << 32 | sg)) - (int64_t)(int32_t)sg;
-        l[k] = (int32_t)(uint32_t)x;
-        h[k] = (int32_t)(x >> 32) + (int32_t)((uint32_t)l[k] >> 31);
-    }
+    for (int k = 0; k < 6; k++) fx_limbs(v[2 * k], v[2 * k + 1], t, BACK ? 0xffffffffu : 0u, h[k], l[k]);
     // the component that enters with both signs, negated: im forward, re backward
 #pragma unroll
-    for (int j = 0; j < 3; j++) {
-        // (-2^31 has no negative in 32 bits: its limb is -(2^31 - 1), one unit of 2^-60 off)
-        nh[j] = -h[2 * j + (BACK ? 0 : 1)];
-        nl[j] = max(-2147483647, l[2 * j + (BACK ? 0 : 1)]);
-        nl[j] = -nl[j];
-    }
+    for (int j = 0; j < 3; j++) fx_neg(h[2 * j + (BACK ? 0 : 1)], l[2 * j + (BACK ? 0 : 1)], nh[j], nl[j]);
 #pragma unroll
     for (int i = 0; i < 3; i++)
 #pragma unroll
@@ -228,14 +234,14 @@ __device__ __forceinline__ void fx_combine(FxAcc &a)
     }
 }
 
-// component k as a double, to nearest, on integers: FP64 operations (four per component with exact
+// (H 2^32 + M) 2^(E - 2132) as a double, to nearest, on integers: FP64 operations (four per component with exact
 // splittings of the words) took 13 % of the normal operator's time at 2 a clock and SM
-__device__ __forceinline__ double fx_value(const FxAcc &a, int k)
+__device__ __forceinline__ double fx_value(int64_t H, uint32_t M, uint32_t E)
 {
     // magnitude of the 96-bit sum H 2^32 + M as words x2 x1 x0
-    const uint32_t sg = (uint32_t)((int32_t)(a.H[k] >> 32) >> 31);
-    uint32_t x0 = (uint32_t)a.M[k] ^ sg;
-    uint64_t xh = (uint64_t)a.H[k] ^ ((uint64_t)sg << 32 | sg);
+    const uint32_t sg = (uint32_t)((int32_t)(H >> 32) >> 31);
+    uint32_t x0 = M ^ sg;
+    uint64_t xh = (uint64_t)H ^ ((uint64_t)sg << 32 | sg);
     xh += (uint64_t)(sg & (uint32_t)(x0 == 0xffffffffu)); // + 1, carried
     x0 -= sg;
     uint32_t x2 = (uint32_t)(xh >> 32), x1 = (uint32_t)xh;
@@ -251,11 +257,12 @@ __device__ __forceinline__ double fx_value(const FxAcc &a, int k)
     const int lz = __clz((int)x2);
     const uint32_t m1 = __funnelshift_l(x1, x2, lz), m0 = __funnelshift_l(x0, x1, lz); // leading bit on top
     // (the leading bit adds one to the exponent field, a carry of the rounding another)
-    const int e = (int)a.E + top - lz - 2132 + 1023 - 1;
+    const int e = (int)E + top - lz - 2132 + 1023 - 1;
     uint64_t m = (uint64_t)(m1 >> 11) << 32 | __funnelshift_r(m0, m1, 11);
     m += (m0 >> 10) & 1u;
     m += (uint64_t)((uint32_t)e << 20 | (sg & 0x80000000u)) << 32;
     return x2 ? __longlong_as_double((long long)m) : 0.0;
 }
+__device__ __forceinline__ double fx_value(const FxAcc &a, int k) { return fx_value(a.H[k], (uint32_t)a.M[k], a.E); }
 
 }  // namespace hisq

@@ -10,7 +10,8 @@
 //   S3 = sum_nu stap_nu[F];  S5 = sum_rho stap_rho[sum_{nu != rho} stap_nu[F]];
 //   S7 = sum_sig stap_sig[sum_{rho != sig} stap_rho[sum_{nu != rho, sig} stap_nu[F]]];
 //   L  = the staples whose detour is two steps along nu
-// (all directions different from mu).  Everything is FP64.
+// (all directions different from mu).  Everything is FP64, the products of three matrices in 60-bit
+// fixed point (fixed.cuh): the FP64 pipe, two operations a clock and SM, would bound them.
 // The projection uses the scaled Newton iteration for the polar decomposition,
 //   X <- (g X + X^{-+} / g) / 2,  g = (|X^-1|_F / |X|_F)^(1/2)
 // (N. J. Higham, "Computing the polar decomposition - with applications", SIAM J. Sci. Stat.
@@ -18,6 +19,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "fixed.cuh"
 #include "internal.cuh"
 
 namespace hisq {
@@ -161,34 +163,202 @@ __device__ __forceinline__ uint32_t at(const Lat &L, const int (&c)[4], int d, i
     return site_index(L, y);
 }
 
-// matrix i of a field of V matrices (coherent loads: a launch may read what the one before wrote)
+// Matrix i of a field in work: blocks of 32 matrices, 16-byte chunk q of all of them contiguous (whole
+// 144-byte records would make every load of a warp touch 32 lines).  Coherent loads: a launch may read
+// what the one before wrote.
+__device__ __forceinline__ const double2 *slot(const double2 *f, size_t i) { return f + (i >> 5) * 288 + (i & 31); }
 __device__ __forceinline__ M3 load(const double2 *f, size_t i)
 {
-    const double2 *p = f + i * 9;
+    const double2 *p = slot(f, i);
     M3 r;
 #pragma unroll
-    for (int k = 0; k < 9; k++) r.a[k] = p[k];
+    for (int k = 0; k < 9; k++) r.a[k] = p[32 * k];
     return r;
 }
+// CANON: the caller's layout, one 144-byte record after the other
+template <bool CANON = false>
 __device__ __forceinline__ void store(double2 *f, size_t i, const M3 &m)
 {
-    double2 *p = f + i * 9;
+    double2 *p = CANON ? f + i * 9 : const_cast<double2 *>(slot(f, i));
 #pragma unroll
-    for (int k = 0; k < 9; k++) p[k] = m.a[k];
+    for (int k = 0; k < 9; k++) p[(CANON ? 1 : 32) * k] = m.a[k];
+}
+
+// A matrix in fixed point: complex entry q has the limbs h, l of reals 2q and 2q + 1, value
+// (h 2^32 + l) 2^(code - 1023 - 59)
+struct FxM {
+    int32_t h[18], l[18];
+    uint32_t code;
+    __device__ __forceinline__ bool ok() const { return code - 823u <= 400u; } // 2^-200 .. 2^200
+};
+// link i (stored as fx_encode_link leaves it)
+__device__ __forceinline__ FxM load_fx(const double2 *f, size_t i)
+{
+    const uint4 *p = reinterpret_cast<const uint4 *>(slot(f, i));
+    FxM r;
+    r.code = 0;
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        const uint4 v = p[32 * k];
+        r.l[2 * k] = (int32_t)v.x;
+        r.h[2 * k] = (int32_t)v.y;
+        r.l[2 * k + 1] = (int32_t)v.z;
+        r.h[2 * k + 1] = (int32_t)v.w;
+        if (k == 0) r.code = (v.x & 15u) | (v.z & 15u) << 4;
+        if (k == 1) r.code |= (v.x & 15u) << 8;
+    }
+    return r;
+}
+__device__ __forceinline__ FxM to_fx(const M3 &m)
+{
+    FxM r;
+    uint32_t top = 0;
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        top = max(top, (uint32_t)__double2hiint(m.a[k].x) & 0x7fffffffu);
+        top = max(top, (uint32_t)__double2hiint(m.a[k].y) & 0x7fffffffu);
+    }
+    r.code = top >> 20;
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        fx_limbs((uint32_t)__double2loint(m.a[k].x), (uint32_t)__double2hiint(m.a[k].x), r.code, 0u, r.h[2 * k], r.l[2 * k]);
+        fx_limbs((uint32_t)__double2loint(m.a[k].y), (uint32_t)__double2hiint(m.a[k].y), r.code, 0u, r.h[2 * k + 1],
+                 r.l[2 * k + 1]);
+    }
+    return r;
+}
+// link i as doubles
+__device__ __forceinline__ M3 load_link(const double2 *f, size_t i)
+{
+    const uint4 *p = reinterpret_cast<const uint4 *>(slot(f, i));
+    uint4 v[9];
+#pragma unroll
+    for (int k = 0; k < 9; k++) v[k] = p[32 * k];
+    const uint32_t code = (v[0].x & 15u) | (v[0].z & 15u) << 4 | (v[1].x & 15u) << 8;
+    M3 r;
+    if (code - 823u <= 400u) {
+#pragma unroll
+        for (int k = 0; k < 9; k++) // N = h 2^32 + l as the sum's H
+            r.a[k] = make_double2(fx_value((int64_t)(int32_t)v[k].y * 4294967296ll + (int32_t)v[k].x, 0u, code + 1018u),
+                                  fx_value((int64_t)(int32_t)v[k].w * 4294967296ll + (int32_t)v[k].z, 0u, code + 1018u));
+    } else {
+#pragma unroll
+        for (int k = 0; k < 9; k++) r.a[k] = make_double2(fx_decode(v[k].x, v[k].y, code), fx_decode(v[k].z, v[k].w, code));
+    }
+    return r;
+}
+
+// a row of three complex sums: component 2k + c is H 2^32 + M
+struct FxRow {
+    int64_t H[6], M[6];
+};
+// (re, im) of column k += a b with a = (ar, ai), b's limbs given for each of the four products
+__device__ __forceinline__ void mac(int64_t &H, int64_t &M, int32_t ah, int32_t al, int32_t bh, int32_t bl)
+{
+    H += (int64_t)ah * bh;
+    M += (int64_t)ah * bl;
+    M += (int64_t)al * bh;
+}
+__device__ __forceinline__ void fold(FxRow &r)
+{
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        r.H[k] += (int64_t)(int32_t)(r.M[k] >> 32);
+        r.M[k] = (int64_t)(uint32_t)r.M[k];
+    }
+}
+
+// op(A) F op(B) with op the adjoint where DA, DB say so, for codes in range.  Row by row: row i of
+// op(A) F, brought back to two limbs (its sums of six products stay below 2^90.6, 31 bits off leave 2^59.6;
+// the exponent is then cA + cF - 1019), times op(B).
+template <bool DA, bool DB>
+__device__ __forceinline__ M3 product(const FxM &A, const FxM &F, const FxM &B)
+{
+    M3 out;
+    const uint32_t E = A.code + F.code - 1019u + B.code;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        FxRow r = {};
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const int q = DA ? 3 * j + i : 3 * i + j;
+            const int32_t arh = A.h[2 * q], arl = A.l[2 * q], aih = A.h[2 * q + 1], ail = A.l[2 * q + 1];
+            int32_t nh, nl;
+            fx_neg(aih, ail, nh, nl);
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const int f = 2 * (3 * j + k);
+                mac(r.H[2 * k], r.M[2 * k], arh, arl, F.h[f], F.l[f]);
+                mac(r.H[2 * k], r.M[2 * k], DA ? aih : nh, DA ? ail : nl, F.h[f + 1], F.l[f + 1]);
+                mac(r.H[2 * k + 1], r.M[2 * k + 1], arh, arl, F.h[f + 1], F.l[f + 1]);
+                mac(r.H[2 * k + 1], r.M[2 * k + 1], DA ? nh : aih, DA ? nl : ail, F.h[f], F.l[f]);
+            }
+        }
+        fold(r);
+        int32_t ph[6], pl[6];
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+            const int64_t x = (int64_t)((uint64_t)r.H[k] << 1 | (uint32_t)r.M[k] >> 31);
+            pl[k] = (int32_t)(uint32_t)x;
+            ph[k] = (int32_t)(x >> 32) + (int32_t)((uint32_t)pl[k] >> 31);
+        }
+        FxRow o = {};
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            // the part of the row's entry that enters negated: re with B^+, im with B
+            int32_t nh, nl;
+            fx_neg(ph[2 * j + (DB ? 0 : 1)], pl[2 * j + (DB ? 0 : 1)], nh, nl);
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const int b = 2 * (DB ? 3 * k + j : 3 * j + k);
+                mac(o.H[2 * k], o.M[2 * k], ph[2 * j], pl[2 * j], B.h[b], B.l[b]);
+                mac(o.H[2 * k], o.M[2 * k], DB ? ph[2 * j + 1] : nh, DB ? pl[2 * j + 1] : nl, B.h[b + 1], B.l[b + 1]);
+                mac(o.H[2 * k + 1], o.M[2 * k + 1], DB ? nh : ph[2 * j], DB ? nl : pl[2 * j], B.h[b + 1], B.l[b + 1]);
+                mac(o.H[2 * k + 1], o.M[2 * k + 1], ph[2 * j + 1], pl[2 * j + 1], B.h[b], B.l[b]);
+            }
+        }
+        fold(o);
+#pragma unroll
+        for (int k = 0; k < 3; k++)
+            out.a[3 * i + k] = make_double2(fx_value(o.H[2 * k], (uint32_t)o.M[2 * k], E),
+                                            fx_value(o.H[2 * k + 1], (uint32_t)o.M[2 * k + 1], E));
+    }
+    return out;
+}
+
+// the same in FP64, for matrices that the fixed-point range leaves out
+static __device__ __noinline__ void product_f64(bool da, bool db, const double2 *u, size_t ia, size_t ib, M3 &F)
+{
+    const M3 A = load_link(u, ia), B = load_link(u, ib);
+    const M3 P = da ? d_mul(A, F) : mul(A, F);
+    F = db ? mul_d(P, B) : mul(P, B);
+}
+
+// op(A) F op(B) of links ia and ib; get() gives F as doubles, F in fixed point
+template <bool DA, bool DB, class Get>
+__device__ __forceinline__ M3 around(const double2 *u, size_t ia, const FxM &F, size_t ib, const Get &get)
+{
+    const FxM A = load_fx(u, ia), B = load_fx(u, ib);
+    if (A.ok() && B.ok() && F.ok()) return product<DA, DB>(A, F, B);
+    M3 r = get();
+    product_f64(DA, DB, u, ia, ib, r);
+    return r;
 }
 
 // The two halves of stap_nu[F]_mu(x) = up + down for a field of V matrices F (of direction mu):
 //   up   = U_nu(x) F(x+nu) U_nu(x+mu)^+,   down = U_nu(x-nu)^+ F(x-nu) U_nu(x-nu+mu)
-// with Fu, Fd the matrices F(x+nu), F(x-nu).
-__device__ __forceinline__ M3 stap_up(const Lat &L, const double2 *u, int mu, int nu, const int (&x)[4], const M3 &Fu)
+// with get() the matrix F(x+nu) or F(x-nu).
+template <class Get>
+__device__ __forceinline__ M3 stap_up(const Lat &L, const double2 *u, int mu, int nu, const int (&x)[4], const Get &get)
 {
     const size_t o = (size_t)nu * L.V;
-    return mul_d(mul(load(u, o + site_index(L, x)), Fu), load(u, o + at(L, x, mu, 1)));
+    return around<false, true>(u, o + site_index(L, x), to_fx(get()), o + at(L, x, mu, 1), get);
 }
-__device__ __forceinline__ M3 stap_down(const Lat &L, const double2 *u, int mu, int nu, const int (&x)[4], const M3 &Fd)
+template <class Get>
+__device__ __forceinline__ M3 stap_down(const Lat &L, const double2 *u, int mu, int nu, const int (&x)[4], const Get &get)
 {
     const size_t o = (size_t)nu * L.V;
-    return mul(d_mul(load(u, o + at(L, x, nu, -1)), Fd), load(u, o + at(L, x, nu, -1, mu, 1)));
+    return around<true, false>(u, o + at(L, x, nu, -1), to_fx(get()), o + at(L, x, nu, -1, mu, 1), get);
 }
 
 struct Coef {
@@ -204,10 +374,12 @@ struct Coef {
 // direction, so launch 3 only adds cl T_up to what the upper half encloses and cl T_down to the
 // lower: no product of its own.  48 matrix products per link and level; building every path from
 // its links took 252 (300 with Lepage).
-// FP64-bound (48 x 108 FMAs per link at two a clock and SM): one thread per (site, detour) in
-// launches 1 and 2, one per site in 3, all with consecutive sites in consecutive lanes.
-// 24^3 x 8, the whole call with projection and Naik links: 76.0 ms before, 12.4 ms now (7.7 ms
-// is what the FP64 pipe needs for the products).
+// The products run on integers (product): FP64 multiply-adds, 48 x 108 per link at two a clock and SM,
+// took 9.5 of 12.4 ms on 24^3 x 8, 4.9 of 7.6 ms so; what is left is bound by integer and FP64
+// issue at eight warps an SM (the operands of a product fill the registers).  One thread per (site,
+// detour) in launches 1 and 2, one per site in 3, consecutive sites in consecutive lanes.
+// 24^3 x 8, the whole call with projection and Naik links: 76.0 ms with every path multiplied out, 12.4
+// with stored staples in FP64, 7.6 with these products.
 __global__ void __launch_bounds__(128) k_stap3(Lat L, const double2 *u, int mu, double2 *t, double2 *td)
 {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -215,9 +387,11 @@ __global__ void __launch_bounds__(128) k_stap3(Lat L, const double2 *u, int mu, 
     const int n = blockIdx.y, nu = n + (n >= mu);
     int x[4];
     coords(L, i, x);
-    const double2 *f = u + (size_t)mu * L.V * 9;
-    M3 up = stap_up(L, u, mu, nu, x, load(f, at(L, x, nu, 1)));
-    const M3 dn = stap_down(L, u, mu, nu, x, load(f, at(L, x, nu, -1)));
+    const size_t m = (size_t)mu * L.V, o = (size_t)nu * L.V;
+    const size_t iu = m + at(L, x, nu, 1), id = m + at(L, x, nu, -1);
+    M3 up = around<false, true>(u, o + site_index(L, x), load_fx(u, iu), o + at(L, x, mu, 1), [&] { return load_link(u, iu); });
+    const M3 dn = around<true, false>(u, o + at(L, x, nu, -1), load_fx(u, id), o + at(L, x, nu, -1, mu, 1),
+                                      [&] { return load_link(u, id); });
     if (td) store(td, (size_t)n * L.V + i, dn);
     else axpy(up, 1.0, dn);
     store(t, (size_t)n * L.V + i, up);
@@ -244,13 +418,14 @@ __global__ void __launch_bounds__(128) k_stap5(Lat L, const double2 *u, int mu, 
     for (int k = 1; k < 3; k++) {
         const int na = (n + k) % 3, nb = (n + 3 - k) % 3; // the two other detours, in both orders
         const int a = na + (na >= mu);
-        axpy(acc, c.c7, stap_up(L, u, mu, a, x, load_t(L, t, td, nb, at(L, x, a, 1))));
-        axpy(acc, c.c7, stap_down(L, u, mu, a, x, load_t(L, t, td, nb, at(L, x, a, -1))));
+        axpy(acc, c.c7, stap_up(L, u, mu, a, x, [&] { return load_t(L, t, td, nb, at(L, x, a, 1)); }));
+        axpy(acc, c.c7, stap_down(L, u, mu, a, x, [&] { return load_t(L, t, td, nb, at(L, x, a, -1)); }));
         axpy(acc, c.c5, load_t(L, t, td, na, i));
     }
     store(g, (size_t)n * L.V + i, acc);
 }
 
+template <bool CANON>
 __global__ void __launch_bounds__(128) k_stap7(Lat L, const double2 *u, int mu, const double2 *t, const double2 *td,
                                                const double2 *g, double2 *out, Coef c)
 {
@@ -259,24 +434,26 @@ __global__ void __launch_bounds__(128) k_stap7(Lat L, const double2 *u, int mu, 
     int x[4];
     coords(L, i, x);
     M3 acc = zero();
-    axpy(acc, c.c1, load(u, (size_t)mu * L.V + i));
+    axpy(acc, c.c1, load_link(u, (size_t)mu * L.V + i));
 #pragma unroll 1
     for (int n = 0; n < 3; n++) {
         const int rho = n + (n >= mu);
         const uint32_t ju = at(L, x, rho, 1), jd = at(L, x, rho, -1);
-        M3 F = load(g, (size_t)n * L.V + ju);
-        if (td) axpy(F, c.cl, load(t, (size_t)n * L.V + ju));
-        axpy(acc, 1.0, stap_up(L, u, mu, rho, x, F));
-        F = load(g, (size_t)n * L.V + jd);
-        if (td) axpy(F, c.cl, load(td, (size_t)n * L.V + jd));
-        axpy(acc, 1.0, stap_down(L, u, mu, rho, x, F));
+        const auto inner = [&](const double2 *half, uint32_t j) {
+            M3 F = load(g, (size_t)n * L.V + j);
+            if (td) axpy(F, c.cl, load(half, (size_t)n * L.V + j));
+            return F;
+        };
+        axpy(acc, 1.0, stap_up(L, u, mu, rho, x, [&] { return inner(t, ju); }));
+        axpy(acc, 1.0, stap_down(L, u, mu, rho, x, [&] { return inner(td, jd); }));
         axpy(acc, c.c3, load_t(L, t, td, n, i));
     }
-    store(out, (size_t)mu * L.V + i, acc);
+    store<CANON>(out, (size_t)mu * L.V + i, acc);
 }
 
 // One smearing level of the links u into out.  t, td, g: scratch of 3 V matrices each (td NULL: no
-// Lepage paths); none of them overlaps u or out.
+// Lepage paths); none of them overlaps u or out.  CANON: out in the caller's layout.
+template <bool CANON>
 static void smear_level(const Lat &L, const double2 *u, double2 *out, double2 *t, double2 *td, double2 *g, const Coef &c,
                         cudaStream_t st)
 {
@@ -284,7 +461,7 @@ static void smear_level(const Lat &L, const double2 *u, double2 *out, double2 *t
     for (int mu = 0; mu < 4; mu++) {
         k_stap3<<<dim3(nb, 3), 128, 0, st>>>(L, u, mu, t, td);
         k_stap5<<<dim3(nb, 3), 128, 0, st>>>(L, u, mu, t, td, g, c);
-        k_stap7<<<nb, 128, 0, st>>>(L, u, mu, t, td, g, out, c);
+        k_stap7<CANON><<<nb, 128, 0, st>>>(L, u, mu, t, td, g, out, c);
     }
 }
 
@@ -326,15 +503,40 @@ __device__ __forceinline__ double fro2(const M3 &A)
     return s;
 }
 
+// a matrix as a link of the second level (fixed point, in blocks)
+__device__ __forceinline__ void store_link(double2 *f, size_t i, const M3 &m)
+{
+    double d[18];
+    uint32_t w[36];
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        d[2 * k] = m.a[k].x;
+        d[2 * k + 1] = m.a[k].y;
+    }
+    fx_encode_link(d, w);
+    uint4 *p = reinterpret_cast<uint4 *>(const_cast<double2 *>(slot(f, i)));
+#pragma unroll
+    for (int k = 0; k < 9; k++) p[32 * k] = make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
+}
+
+// the caller's thin links (records) as links of the first level
+__global__ void __launch_bounds__(128) k_take_links(const double2 *thin, double2 *u, uint64_t n)
+{
+    const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    if (t >= n) return;
+    M3 m;
+#pragma unroll
+    for (int k = 0; k < 9; k++) m.a[k] = thin[t * 9 + k];
+    store_link(u, t, m);
+}
+
 // W = unitary polar factor of V (scaled Newton iteration); a singular or non-converging
 // matrix raises the device error flag
 __global__ void __launch_bounds__(128) k_project_u3(const double2 *v, double2 *w, uint64_t n, DevStatus *status)
 {
     const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     if (t >= n) return;
-    M3 X;
-#pragma unroll
-    for (int i = 0; i < 9; i++) X.a[i] = v[t * 9 + i];
+    M3 X = load(v, t);
     bool ok = false;
     for (int it = 0; it < 30; it++) {
         M3 Xi;
@@ -361,8 +563,7 @@ __global__ void __launch_bounds__(128) k_project_u3(const double2 *v, double2 *w
             break;
         }
     }
-#pragma unroll
-    for (int i = 0; i < 9; i++) w[t * 9 + i] = X.a[i];
+    store_link(w, t, X);
     if (!ok && status) {
         status->where = 2; // link projection
         atomicExch(&status->error, (int)HISQ_EDEVICE);
@@ -377,11 +578,11 @@ __global__ void __launch_bounds__(128) k_naik(Lat L, const double2 *w, double2 *
     const int mu = blockIdx.y;
     int x[4];
     coords(L, i, x);
-    const double2 *f = w + (size_t)mu * L.V * 9;
-    const M3 r = mul(mul(load(f, i), load(f, at(L, x, mu, 1))), load(f, at(L, x, mu, 1, mu, 1)));
+    const size_t m = (size_t)mu * L.V, j = m + at(L, x, mu, 1);
+    const M3 r = around<false, false>(w, m + i, load_fx(w, j), m + at(L, x, mu, 1, mu, 1), [&] { return load_link(w, j); });
     M3 o = zero();
     axpy(o, cn, r);
-    store(out, (size_t)mu * L.V + i, o);
+    store<true>(out, (size_t)mu * L.V + i, o);
 }
 
 }  // namespace smear
@@ -422,15 +623,20 @@ extern "C" int hisq_smear_links(const int dims[4], const double *thin, double *f
     double2 *xo = links_on_device ? reinterpret_cast<double2 *>(fat) : x;
     double2 *no = links_on_device ? reinterpret_cast<double2 *>(lng) : nk;
     cudaError_t e = cudaMemsetAsync(status, 0, sizeof(DevStatus), st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(u, thin, bytes, links_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st);
+    // links on the host, or not on the 16-byte boundaries that the kernels read, go through v, which
+    // holds nothing yet
+    const bool direct = links_on_device && (reinterpret_cast<uintptr_t>(thin) & 15) == 0;
+    const double2 *src = direct ? reinterpret_cast<const double2 *>(thin) : v;
+    if (e == cudaSuccess && !direct)
+        e = cudaMemcpyAsync(v, thin, bytes, links_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st);
     const unsigned nb = (unsigned)((V + 127) / 128), nb4 = (unsigned)((4 * V + 127) / 128);
     if (e == cudaSuccess) {
         // scratch of a level (three matrices per site each): fields that hold nothing yet or no
         // longer, so no memory beyond the links, the two levels and the results is needed
-        smear::smear_level(L, u, v, w, nullptr, xo, smear::Coef{1.0 / 8, 1.0 / 16, 1.0 / 64, 1.0 / 384, 0.0}, st);
+        smear::k_take_links<<<nb4, 128, 0, st>>>(src, u, 4 * V);
+        smear::smear_level<false>(L, u, v, w, nullptr, xo, smear::Coef{1.0 / 8, 1.0 / 16, 1.0 / 64, 1.0 / 384, 0.0}, st);
         smear::k_project_u3<<<nb4, 128, 0, st>>>(v, w, 4 * V, status);
-        smear::smear_level(L, w, xo, u, v, no, smear::Coef{1.0, 1.0 / 16, 1.0 / 64, 1.0 / 384, -1.0 / 8}, st);
+        smear::smear_level<true>(L, w, xo, u, v, no, smear::Coef{1.0, 1.0 / 16, 1.0 / 64, 1.0 / 384, -1.0 / 8}, st);
         smear::k_naik<<<dim3(nb, 4), 128, 0, st>>>(L, w, no, -1.0 / 24 + eps_naik / 8);
         e = cudaGetLastError();
     }
