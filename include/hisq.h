@@ -115,8 +115,8 @@ const char *hisq_strerror(int status);
 long hisq_half_volume(const hisq_ctx *ctx);
 
 /* ------------------------------------------------------------------ internal-layout fields */
-/* A field holds nrhs half-lattice vectors in a precision's internal layout (site-major,
- * 16-byte aligned).  It exists so that reduced-precision operators can be applied and
+/* A field holds nrhs half-lattice vectors in a precision's internal layout
+ * (16-byte aligned).  It exists so that reduced-precision operators can be applied and
  * timed without per-call conversions. */
 typedef struct hisq_field hisq_field;
 

@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(128) k_project_u3(const double2 *v, double2 *w
         if (!inverse(X, Xi)) break;
         // any positive g leaves the polar factor alone (it only speeds up the first steps), so its
         // roots and inverse are taken in FP32, and left out once X is close to unitary: with a division
-        // by g for each of the 18 reals the projection took 2.0 ms on 24^3 x 8, 1.0 ms so
+        // by g for each of the 18 reals the projection took 2.0 ms on 24^3 x 8, 1.1 ms so
         double g = 1.0, gi = 1.0;
         if (scaled) {
             const double q = fro2(Xi) / fro2(X);
