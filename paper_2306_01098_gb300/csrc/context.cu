@@ -110,6 +110,7 @@ __global__ void k_import_links(const ImportArgs a)
         const double *L = a.src[type] + ((size_t)mu * V + (size_t)p * a.g.Vh + s) * 18;
         if (a.fixed) {
             double d[18];
+#pragma unroll
             for (int i = 0; i < 18; i++) d[i] = sg * L[i];
             fx_encode_link(d, w);
         } else for (int i = 0; i < a.nreal; i++) {

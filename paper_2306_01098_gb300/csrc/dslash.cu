@@ -81,11 +81,18 @@ static int default_order(hisq_ctx *ctx, int pv, int nrhs)
     return ctx->g.zt_ok && nrhs > 1 && (size_t)nrhs * ctx->g.VhPad * spinor_bytes(pv) > (64u << 20) ? 1 : 0;
 }
 
+// threads per site: FP64 sites keep the SMs busy at 512 threads each (32^3 x 8: 64 us with one thread per
+// site, 66 with two), the others gain from more requests in flight up to larger lattices
+int default_ds(const hisq_ctx *ctx, int pv)
+{
+    return ctx->g.Vh < (pv == HISQ_F64 ? 512u * (uint32_t)ctx->sm_count : 1u << 20) ? 2 : 1;
+}
+
 static DslashShape default_shape(hisq_ctx *ctx, int pv, int nrhs)
 {
     DslashShape s;
     s.nr = ctx->batch ? 1 : pick_inner(pv, nrhs);
-    s.ds = ctx->g.Vh < (1u << 20) ? 2 : 1;
+    s.ds = default_ds(ctx, pv);
     s.order = default_order(ctx, pv, nrhs);
     return s;
 }

@@ -55,6 +55,7 @@ cudaError_t dslash_launch(int pl, int pv, int epi, const DslashArgs &a, int nrea
 DslashShape dslash_shape(hisq_ctx *ctx, int pl, int pv, int nrhs, const void *in, void *out, size_t rhs_bytes,
                          cudaStream_t st);
 int pick_inner(int prec, int nrhs);
+int default_ds(const hisq_ctx *ctx, int pv);
 
 #define HISQ_DSLASH_DECLARE(PL, PV) \
     cudaError_t dslash_launch_##PL##_##PV(int epi, const DslashArgs &a, int nreal, int nr, int ds, int rg,      \

@@ -346,10 +346,11 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const Geom &g, 
     using TL = Prec<PL>; // link storage
     constexpr int LB = NREAL == 18 ? LinkBytes<PL>::b18 : LinkBytes<PL>::b12;
     constexpr bool TWO = (PL == HISQ_F16 || PL == HISQ_BF16 || NREAL == 12);
-    // directions summed apart: always for float pairs; for FP32 with one right-hand side, so that a
-    // site's error does not depend on how many threads share it (measured 1.9e-7 with one running sum,
-    // 1.2e-7 apart; the gathers hide the 24 additions)
-    constexpr bool SPLIT = T::kSplitDirections || (PL == HISQ_F32 && NR == 1 && !TWO && !COH && DS < 4);
+    // directions summed apart: always for float pairs; for FP32 with one or four right-hand sides (with
+    // two, the registers would cost more than the additions: 14 shifts, FP32 32^3 x 8, 60 -> 67 ms), so that
+    // a site's error depends less on how many threads share it (measured 1.9e-7 with one running
+    // sum, 1.2e-7 apart; the gathers hide the 24 additions)
+    constexpr bool SPLIT = T::kSplitDirections || (PL == HISQ_F32 && (NR == 1 || NR == 4) && !TWO && !COH && DS < 4);
     constexpr int NMU = 4 / DS;
     const uint32_t gt = tile * (uint32_t)a.bs + tid;
     // site number in launch order, and this thread's directions: with DS > 1 a warp holds 32 / DS
@@ -578,11 +579,12 @@ __device__ __forceinline__ double dot_value(double x) { return x; }
 // 256-thread blocks per SM that the registers are limited for.  Left alone the compiler moves the
 // loads of all 16 hops to the front of the site (250 registers, 8 warps an SM); the gathers want warps:
 // FP32 vectors 48 / 64 / 128 registers at 1 / 2 / 4 right-hand sides a thread (14-shift FP32 solve
-// 32^3 x 8: 74 ms without limits, 63 ms with 64 / 80 / 128, 59 ms so), FP64 and float pairs 128 at one.
+// 32^3 x 8: 74 ms without limits, 63 ms with 64 / 80 / 128, 59 ms so; one block less for rebuilt third
+// rows), FP64 and float pairs 128 at one.
 constexpr int min_blocks(int pl, int pv, int nreal, int nr)
 {
     if (pv == HISQ_F64 || pv == HISQ_F64X) return nr == 1 && !(pl == HISQ_F64 && nreal == 12) ? 2 : 1;
-    const int less = nreal == 12 ? 1 : 0; // (the rebuilt third row)
+    const int less = nreal == 12 ? 1 : 0;
     return nr == 1 ? 5 - less : nr == 2 ? 4 - less : nr == 4 ? 2 : 1;
 }
 template <int PL, int PV, int NREAL, int NR, int EPI, int DS, bool BATCH, int RG = 1, int WG = 1>

@@ -16,11 +16,12 @@
 // Errors of a site, relative to the largest |link| |vector| among its hops: 2^-61 (vector) and
 // 2^-61 (link; 2^-57 for the three entries that carry the exponent) per product, against 2^-53
 // per product and per sum in FP64; the sum is rounded to FP64 once.
-// Measured (max over a field, relative to its largest entry): 2.5e-16 after the normal operator of a
+// Measured (max over a field, relative to its largest entry): 2.4e-16 after the normal operator of a
 // 32^3 x 8 lattice, 3.9e-16 with FP64 multiply-adds.  Time there, two Dslash launches: 280.8 us with
-// FP64 multiply-adds (their pipe alone needs 250 us), 147.2 us so (the bytes need 93 us).
-// Sites that meet anything this cannot hold (an infinity or NaN, or values below about 1e-280 or
-// products beyond about 1e+-280) are computed in FP64 instead (fx_site_f64).
+// FP64 multiply-adds (their pipe alone needs 250 us), 131 us so (the bytes need 93 us).
+// Sites that meet anything this cannot hold (an infinity or NaN, a link or vector whose largest real is
+// below about 1e-289, products outside about 1e-254 .. 1e287) are computed in FP64 instead
+// (fx_site_f64).
 #pragma once
 
 #include "internal.cuh"
@@ -42,6 +43,7 @@ __host__ __device__ inline void fx_encode_link(const double (&d)[18], uint32_t (
     uint64_t b[18];
     uint32_t em = 0;
     bool zero = true;
+#pragma unroll
     for (int i = 0; i < 18; i++) {
         union { double d; uint64_t u; } c;
         c.d = d[i];
@@ -52,6 +54,7 @@ __host__ __device__ inline void fx_encode_link(const double (&d)[18], uint32_t (
     }
     const bool raw = !zero && (em < kFxMinExp || em == 0x7ffu);
     const uint32_t code = zero ? 0u : raw ? kFxRaw : em;
+#pragma unroll
     for (int i = 0; i < 18; i++) {
         const int64_t nib = i < 3 ? (int64_t)((code >> (4 * i)) & 15u) : 0;
         if (raw) {

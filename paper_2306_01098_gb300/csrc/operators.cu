@@ -36,7 +36,7 @@ int apply_mdagm(hisq_ctx *ctx, int prec, double m, const void *in, void *tmp, vo
     } else {
         auto it = ctx->tune.find(tune_key(prec, pv, nrhs));
         sh.nr = it != ctx->tune.end() ? it->second.nr : pick_inner(pv, nrhs);
-        sh.ds = it != ctx->tune.end() ? it->second.ds : (ctx->g.Vh < (1u << 20) ? 2 : 1);
+        sh.ds = it != ctx->tune.end() ? it->second.ds : default_ds(ctx, pv);
         sh.order = it != ctx->tune.end() ? it->second.order : 0;
         sh.bs = it != ctx->tune.end() ? it->second.bs : kDslashBlock;
         sh.rg = it != ctx->tune.end() ? it->second.rg : 1;
