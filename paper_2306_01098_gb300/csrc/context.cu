@@ -112,7 +112,9 @@ __global__ void k_import_links(const ImportArgs a)
             double d[18];
 #pragma unroll
             for (int i = 0; i < 18; i++) d[i] = sg * L[i];
-            fx_encode_link(d, w);
+            uint64_t rest;
+            fx_encode_link(d, w, rest);
+            reinterpret_cast<uint64_t *>(dst + (size_t)a.g.VhPad * LB)[s] = rest;
         } else for (int i = 0; i < a.nreal; i++) {
             const double d = sg * L[i];
             switch (a.prec) {
@@ -310,7 +312,8 @@ static int build_store(hisq_ctx *ctx, int prec, int nreal, const double *fat, co
     LinkStore &L = ctx->links[prec];
     const int LB = link_bytes(prec, nreal);
     L.nreal = nreal;
-    L.slot_bytes = (size_t)ctx->g.VhPad * LB;
+    const bool fixed = prec == HISQ_F64 && nreal == 18 && !ctx->links_double;
+    L.slot_bytes = (size_t)ctx->g.VhPad * (LB + (fixed ? kFxRestBytes : 0));
     cudaError_t e = cudaMalloc((void **)&L.base, L.slot_bytes * kSlots);
     if (e != cudaSuccess) return cuda_error(ctx, e, "link store allocation");
     ImportArgs a{};
@@ -322,7 +325,7 @@ static int build_store(hisq_ctx *ctx, int prec, int nreal, const double *fat, co
     a.prec = prec;
     a.nreal = nreal;
     a.phased = ctx->links_phased;
-    a.fixed = prec == HISQ_F64 && nreal == 18 && !ctx->links_double;
+    a.fixed = fixed;
     for (int t = 0; t < 2; t++) {
         double sc = 1.0;
         if (nreal == 12) sc = c[t];

@@ -236,13 +236,13 @@ static __device__ __noinline__ void fx_site_f64(const DslashArgs &a, const Geom 
         const uint32_t sn = neighbour(g, c, s, mu, back ? -k : k, wrap);
         const int lp = back ? 1 - a.p : a.p;
         uint32_t w[36];
-        load_link_words<144>(links + (size_t)((lp * 2 + type) * 4 + mu) * slot_bytes, back ? sn : s, w);
-        const uint32_t code = fx_code(w);
+        const char *slot = links + (size_t)((lp * 2 + type) * 4 + mu) * slot_bytes;
+        load_link_words<144>(slot, back ? sn : s, w);
+        const uint64_t rest = reinterpret_cast<const uint64_t *>(slot + (size_t)g.VhPad * 144)[back ? sn : s];
         Prec<HISQ_F64>::Link U;
         Prec<HISQ_F64>::Vec v;
         Prec<HISQ_F64>::Acc acc;
-#pragma unroll
-        for (int i = 0; i < 18; i++) U.v[i] = fx_decode(w[2 * i], w[2 * i + 1], code);
+        fx_decode_link(w, rest, U.v);
 #pragma unroll
         for (int i = 0; i < 6; i++) acc.v[i] = out[i];
         Prec<HISQ_F64>::load(in, sn, v);
@@ -276,7 +276,7 @@ __device__ __forceinline__ void fx_site(const DslashArgs &a, const Geom &g, cons
             for (int h = 0; h < 4; h++) {
                 uint32_t w[36];
                 pipe.link(h, w);
-                const uint32_t code = fx_code(w);
+                const uint32_t code = fx_take_code(w);
 #pragma unroll
                 for (int r = 0; r < NR; r++) {
                     uint32_t x[12];

@@ -7,97 +7,148 @@
 //   a link is  Lambda 2^(e_L - 59),   Lambda integer, |Lambda| <= 2^60, 2^e_L <= max |entry| < 2^(e_L + 1)
 //   a vector is     N 2^(e_v - 59)    likewise, made from its doubles when it is loaded
 // both kept as two limbs, x = h 2^32 + l with -2^31 <= l < 2^31 and |h| <= 2^28.  A product is
-//   h h' 2^64 + (h l' + l h') 2^32     (l l' is dropped: at most 2^-58 of max |entry| max |v|)
+//   h h' 2^64 + (h l' + l h') 2^32     (l l' is dropped: at most 2^62 of up to 2^120)
 // i.e. three multiply-adds into two 64-bit sums, H and M.  Bounds: H adds 96 products of at most
 // 2^56 per component and site (16 hops, 3 colours, re and im): < 2^62.6.  M adds 12 products of
 // at most 2^59 per hop, and is folded into H after every hop: < 2^62.6 too.  Nothing is lost in
 // the sums; all hops of a site are aligned to the largest exponent e_L + e_v met so far (H and M
 // are shifted when a larger one comes).
-// Errors of a site, relative to the largest |link| |vector| among its hops: 2^-61 (vector) and
-// 2^-61 (link; 2^-57 for the three entries that carry the exponent) per product, against 2^-53
-// per product and per sum in FP64; the sum is rounded to FP64 once.
+// Error of one real product, in units of 2^(e_L + e_v): 2^-56 for l l', 2^-58 each for the cut of the vector
+// and of the link (one unit of 2^-59, against less than 2), 2^-58 where a limb of -2^31 was negated; the sum is
+// rounded to FP64 once.
 // Measured (max over a field, relative to its largest entry): 2.4e-16 after the normal operator of a
 // 32^3 x 8 lattice, 3.9e-16 with FP64 multiply-adds.  Time there, two Dslash launches: 280.8 us with
 // FP64 multiply-adds (their pipe alone needs 250 us), 131 us so (the bytes need 93 us).
 // Sites that meet anything this cannot hold (an infinity or NaN, a link or vector whose largest real is
-// below about 1e-289, products outside about 1e-254 .. 1e287) are computed in FP64 instead
-// (fx_site_f64).
+// below about 1e-289, products outside about 1e-254 .. 1e287, a link whose reals lie too far apart) are
+// computed in FP64 instead (fx_site_f64), from the same doubles.
 #pragma once
 
 #include "internal.cuh"
 
 namespace hisq {
 
-// Stored link, 18 reals: word 2i the low limb, 2i + 1 the high limb of real i.  The low four bits
-// of the low limbs of reals 0, 1, 2 hold the biased exponent e_L + 1023 (the value is rounded to
-// the nearest one with these bits): 0 for a link of zeros, kFxRaw for one that the format cannot
-// hold, whose words are then the doubles themselves.
-constexpr uint32_t kFxRaw = 0xfff;
-constexpr uint32_t kFxMinExp = 64; // smallest biased exponent of a link or vector in fixed point
+// Stored link, 18 reals: word 2i the low limb of real i, word 2i + 1 its high limb in 30 bits.  The top two
+// bits of the high words of reals 0 .. 5 hold, from real 0 on, the biased exponent e_L + 1023: 0 for a link
+// of zeros, 0x7ff for one that the format cannot hold (an infinity or NaN, entries too small or too far
+// apart), whose words are then the doubles themselves.  Magnitudes are cut, not rounded, to units of
+// 2^(e_L - 59), so that a real's position below e_L can be read off its leading bit, and what was cut is
+// kept: the store holds 64 more bits for every link, `rest`, with the mantissa bits below the unit, real after
+// real (a real 2^-k of the largest has lost its lowest k - 7), or the two bits of each high word that a
+// link of doubles gave to the exponent.  The doubles can be had back exactly (fx_decode_link), zeros stay zeros.
+constexpr uint32_t kFxRaw = 0xfff;  // fx_take_code of a link of doubles
+constexpr uint32_t kFxMinExp = 64;  // smallest biased exponent of a link or vector in fixed point
+constexpr int kFxRestBytes = 8;     // bytes of `rest` per link
 // biased exponents of products (sum of two biased exponents) that the sums are formed with
 // (results, whose last bit is 2^-85 of the largest product, stay normal numbers)
 constexpr uint32_t kFxELo = 1200, kFxEHi = 3000;
 
-__host__ __device__ inline void fx_encode_link(const double (&d)[18], uint32_t (&w)[36])
+__host__ __device__ __forceinline__ uint64_t fx_bits(double x)
 {
-    uint64_t b[18];
+    union { double d; uint64_t u; } c;
+    c.d = x;
+    return c.u;
+}
+// position of the leading bit of x != 0
+__host__ __device__ __forceinline__ int fx_top(uint64_t x)
+{
+#ifdef __CUDA_ARCH__
+    return 63 - __clzll((long long)x);
+#else
+    return 63 - __builtin_clzll(x);
+#endif
+}
+
+__host__ __device__ inline void fx_encode_link(const double (&d)[18], uint32_t (&w)[36], uint64_t &rest)
+{
     uint32_t em = 0;
     bool zero = true;
 #pragma unroll
     for (int i = 0; i < 18; i++) {
-        union { double d; uint64_t u; } c;
-        c.d = d[i];
-        b[i] = c.u;
-        const uint32_t e = (uint32_t)(b[i] >> 52) & 0x7ffu;
+        const uint64_t b = fx_bits(d[i]);
+        const uint32_t e = (uint32_t)(b >> 52) & 0x7ffu;
         em = e > em ? e : em;
-        zero = zero && (b[i] << 1) == 0;
+        zero = zero && (b << 1) == 0;
     }
-    const bool raw = !zero && (em < kFxMinExp || em == 0x7ffu);
-    const uint32_t code = zero ? 0u : raw ? kFxRaw : em;
+    bool raw = !zero && (em < kFxMinExp || em == 0x7ffu);
+    uint32_t used = 0;
+    rest = 0;
 #pragma unroll
     for (int i = 0; i < 18; i++) {
-        const int64_t nib = i < 3 ? (int64_t)((code >> (4 * i)) & 15u) : 0;
-        if (raw) {
-            const uint64_t x = i < 3 ? (b[i] & ~15ull) | (uint64_t)nib : b[i];
-            w[2 * i] = (uint32_t)x;
-            w[2 * i + 1] = (uint32_t)(x >> 32);
-            continue;
-        }
-        // 53-bit magnitude, shifted left by 7 (60 bits) and right by the distance to the
-        // largest exponent, to nearest
-        const uint32_t e = (uint32_t)(b[i] >> 52) & 0x7ffu, s = em - e;
+        const uint64_t b = fx_bits(d[i]);
+        const uint32_t e = (uint32_t)(b >> 52) & 0x7ffu, s = em - e;
         int64_t x = 0;
-        if (e != 0 && s < 62) {
-            const int64_t m = (int64_t)(((b[i] & 0xfffffffffffffull) | 0x10000000000000ull) << 7);
-            x = (m + (s ? (int64_t)1 << (s - 1) : 0)) >> s;
-            if (b[i] >> 63) x = -x;
+        if ((b << 1) != 0 && !raw) {
+            // 53-bit magnitude, shifted left by 7 (60 bits) and right by the distance to the largest exponent
+            const uint64_t m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 7;
+            const uint32_t n = s > 7 ? s - 7 : 0;
+            if (e == 0 || s > 59 || used + n > 64) {
+                raw = true;
+            } else {
+                if (n) rest |= ((m & ((1ull << s) - 1)) >> 7) << used;
+                used += n;
+                x = (int64_t)(m >> s);
+                if (b >> 63) x = -x;
+            }
         }
-        if (i < 3) x = ((x - nib + 8) & ~(int64_t)15) + nib;
         const int32_t l = (int32_t)(uint32_t)x;
         w[2 * i] = (uint32_t)l;
         w[2 * i + 1] = (uint32_t)((x - l) >> 32);
     }
-}
-
-// biased exponent of a stored link
-__host__ __device__ __forceinline__ uint32_t fx_code(const uint32_t (&w)[36])
-{
-    return (w[0] & 15u) | (w[2] & 15u) << 4 | (w[4] & 15u) << 8;
-}
-
-// the link as doubles (fallback and tests)
-__host__ __device__ inline double fx_decode(uint32_t lo, uint32_t hi, uint32_t code)
-{
-    union { double d; uint64_t u; } c;
-    if (code == kFxRaw) {
-        c.u = (uint64_t)hi << 32 | lo;
-        return c.d;
+    const uint32_t code = zero ? 0u : raw ? 0x7ffu : em;
+    if (raw) rest = 0;
+#pragma unroll
+    for (int i = 0; i < 18; i++) {
+        if (raw) {
+            const uint64_t b = fx_bits(d[i]);
+            w[2 * i] = (uint32_t)b;
+            w[2 * i + 1] = (uint32_t)(b >> 32);
+            if (i < 6) rest |= (uint64_t)(w[2 * i + 1] >> 30) << (2 * i);
+        }
+        if (i < 6) w[2 * i + 1] = (w[2 * i + 1] & 0x3fffffffu) | ((code >> (2 * i)) & 3u) << 30;
     }
-    if (code == 0) return 0.0;
-    // 2^(code - 1023 - 59) as a product of two powers (either may leave the normal range alone)
-    c.u = (uint64_t)code << 52;
-    const double x = (double)((int64_t)(int32_t)hi * 4294967296ll + (int32_t)lo);
-    return x * 1.734723475976807e-18 * c.d; // 2^-59
+}
+
+// biased exponent of a stored link (kFxRaw: doubles, which stay as stored); the words become the limbs
+__host__ __device__ __forceinline__ uint32_t fx_take_code(uint32_t (&w)[36])
+{
+    uint32_t code = 0;
+#pragma unroll
+    for (int i = 5; i >= 0; i--) {
+        code = code << 2 | w[2 * i + 1] >> 30;
+        w[2 * i + 1] = (uint32_t)((int32_t)(w[2 * i + 1] << 2) >> 2);
+    }
+    return code == 0x7ffu ? kFxRaw : code;
+}
+
+// the doubles of a stored link (its words as stored)
+__host__ __device__ inline void fx_decode_link(const uint32_t (&w)[36], uint64_t rest, double (&d)[18])
+{
+    uint32_t code = 0;
+#pragma unroll
+    for (int i = 0; i < 6; i++) code |= (w[2 * i + 1] >> 30) << (2 * i);
+    uint32_t used = 0;
+#pragma unroll
+    for (int i = 0; i < 18; i++) {
+        union { double d; uint64_t u; } c;
+        if (code == 0x7ffu) {
+            const uint32_t hi = i < 6 ? (w[2 * i + 1] & 0x3fffffffu) | ((uint32_t)(rest >> (2 * i)) & 3u) << 30 : w[2 * i + 1];
+            c.u = (uint64_t)hi << 32 | w[2 * i];
+        } else {
+            const int32_t h = i < 6 ? (int32_t)(w[2 * i + 1] << 2) >> 2 : (int32_t)w[2 * i + 1];
+            const int64_t x = (int64_t)h * 4294967296ll + (int32_t)w[2 * i];
+            const uint64_t a = (uint64_t)(x < 0 ? -x : x);
+            c.u = 0;
+            if (a) {
+                const uint32_t s = 59u - (uint32_t)fx_top(a), n = s > 7 ? s - 7 : 0;
+                uint64_t m = a << s;
+                if (n) m |= ((rest >> used) & ((1ull << n) - 1)) << 7;
+                used += n;
+                c.u = (x < 0 ? 1ull << 63 : 0ull) | (uint64_t)(code - s) << 52 | ((m >> 7) & 0xfffffffffffffull);
+            }
+        }
+        d[i] = c.d;
+    }
 }
 
 // running sums of one output vector: component k is (H[k] 2^32 + M[k]) 2^(E - 2046 - 118 + 32)
@@ -159,8 +210,8 @@ __device__ __forceinline__ void fx_neg(int32_t h, int32_t l, int32_t &nh, int32_
     nl = -max(-2147483647, l);
 }
 
-// a += U v (BACK = false) or a -= U^+ v (BACK = true); w: the stored link, code: its exponent,
-// v: the words of the vector's six doubles
+// a += U v (BACK = false) or a -= U^+ v (BACK = true); w: the link's limbs, code: its exponent
+// (fx_take_code), v: the words of the vector's six doubles
 template <bool BACK>
 __device__ __forceinline__ void fx_hop(FxAcc &a, const uint32_t (&w)[36], uint32_t code, const uint32_t (&v)[12])
 {
@@ -169,11 +220,12 @@ __device__ __forceinline__ void fx_hop(FxAcc &a, const uint32_t (&w)[36], uint32
     for (int k = 0; k < 6; k++) top = max(top, v[2 * k + 1] & 0x7fffffffu);
     const uint32_t ev = top >> 20, e = code ? code + ev : 0u;
     if (ev - kFxMinExp >= 0x7ffu - kFxMinExp || e - kFxELo > kFxEHi - kFxELo) {
-        // zeros contribute nothing; anything else here is left to FP64
+        // a link of zeros, or a vector of zeros unless the link holds doubles (an infinity or NaN among them,
+        // maybe), contributes nothing; anything else here is left to FP64
         uint32_t any = 0;
 #pragma unroll
         for (int k = 0; k < 6; k++) any |= (v[2 * k + 1] & 0x7fffffffu) | v[2 * k];
-        a.bad |= any != 0 && (code != 0 || ev == 0x7ffu);
+        a.bad |= code == kFxRaw || (any != 0 && (code != 0 || ev == 0x7ffu));
         return;
     }
     if (e > a.E) {

@@ -187,7 +187,7 @@ __device__ __forceinline__ size_t link_tail_off(uint32_t s, int LB, int tb)
 
 struct LinkStore {
     char *base = nullptr;   // 16 slots
-    size_t slot_bytes = 0;  // VhPad * link bytes
+    size_t slot_bytes = 0;  // VhPad * link bytes (fixed point: and 8 bytes per link behind them, fixed.cuh)
     int nreal = 0;          // 18 or 12
     int built = 0;
     double scale[2] = {1.0, 1.0}; // multiply the stored link by this (per type): 12-real c,

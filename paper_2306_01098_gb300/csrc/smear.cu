@@ -191,21 +191,31 @@ struct FxM {
     uint32_t code;
     __device__ __forceinline__ bool ok() const { return code - 823u <= 400u; } // 2^-200 .. 2^200
 };
-// link i (stored as fx_encode_link leaves it)
-__device__ __forceinline__ FxM load_fx(const double2 *f, size_t i)
+// A field of links holds them as fx_encode_link leaves them, the `rest` of link i behind all of them.
+__device__ __forceinline__ void link_words(const double2 *f, size_t i, uint32_t (&w)[36])
 {
     const uint4 *p = reinterpret_cast<const uint4 *>(slot(f, i));
-    FxM r;
-    r.code = 0;
 #pragma unroll
     for (int k = 0; k < 9; k++) {
         const uint4 v = p[32 * k];
-        r.l[2 * k] = (int32_t)v.x;
-        r.h[2 * k] = (int32_t)v.y;
-        r.l[2 * k + 1] = (int32_t)v.z;
-        r.h[2 * k + 1] = (int32_t)v.w;
-        if (k == 0) r.code = (v.x & 15u) | (v.z & 15u) << 4;
-        if (k == 1) r.code |= (v.x & 15u) << 8;
+        w[4 * k] = v.x;
+        w[4 * k + 1] = v.y;
+        w[4 * k + 2] = v.z;
+        w[4 * k + 3] = v.w;
+    }
+}
+__device__ __forceinline__ const uint64_t *rests(const double2 *f, uint32_t V) { return reinterpret_cast<const uint64_t *>(f + (size_t)36 * V); }
+// link i of a field
+__device__ __forceinline__ FxM load_fx(const double2 *f, size_t i)
+{
+    uint32_t w[36];
+    link_words(f, i, w);
+    FxM r;
+    r.code = fx_take_code(w);
+#pragma unroll
+    for (int k = 0; k < 18; k++) {
+        r.l[k] = (int32_t)w[2 * k];
+        r.h[k] = (int32_t)w[2 * k + 1];
     }
     return r;
 }
@@ -227,24 +237,16 @@ __device__ __forceinline__ FxM to_fx(const M3 &m)
     }
     return r;
 }
-// link i as doubles
-__device__ __forceinline__ M3 load_link(const double2 *f, size_t i)
+// link i of a field of 4 V links as doubles
+__device__ __forceinline__ M3 load_link(const double2 *f, uint32_t V, size_t i)
 {
-    const uint4 *p = reinterpret_cast<const uint4 *>(slot(f, i));
-    uint4 v[9];
-#pragma unroll
-    for (int k = 0; k < 9; k++) v[k] = p[32 * k];
-    const uint32_t code = (v[0].x & 15u) | (v[0].z & 15u) << 4 | (v[1].x & 15u) << 8;
+    uint32_t w[36];
+    double d[18];
+    link_words(f, i, w);
+    fx_decode_link(w, rests(f, V)[i], d);
     M3 r;
-    if (code - 823u <= 400u) {
 #pragma unroll
-        for (int k = 0; k < 9; k++) // N = h 2^32 + l as the sum's H
-            r.a[k] = make_double2(fx_value((int64_t)(int32_t)v[k].y * 4294967296ll + (int32_t)v[k].x, 0u, code + 1018u),
-                                  fx_value((int64_t)(int32_t)v[k].w * 4294967296ll + (int32_t)v[k].z, 0u, code + 1018u));
-    } else {
-#pragma unroll
-        for (int k = 0; k < 9; k++) r.a[k] = make_double2(fx_decode(v[k].x, v[k].y, code), fx_decode(v[k].z, v[k].w, code));
-    }
+    for (int k = 0; k < 9; k++) r.a[k] = make_double2(d[2 * k], d[2 * k + 1]);
     return r;
 }
 
@@ -327,21 +329,21 @@ __device__ __forceinline__ M3 product(const FxM &A, const FxM &F, const FxM &B)
 }
 
 // the same in FP64, for matrices that the fixed-point range leaves out
-static __device__ __noinline__ void product_f64(bool da, bool db, const double2 *u, size_t ia, size_t ib, M3 &F)
+static __device__ __noinline__ void product_f64(bool da, bool db, const double2 *u, uint32_t V, size_t ia, size_t ib, M3 &F)
 {
-    const M3 A = load_link(u, ia), B = load_link(u, ib);
+    const M3 A = load_link(u, V, ia), B = load_link(u, V, ib);
     const M3 P = da ? d_mul(A, F) : mul(A, F);
     F = db ? mul_d(P, B) : mul(P, B);
 }
 
 // op(A) F op(B) of links ia and ib; get() gives F as doubles, F in fixed point
 template <bool DA, bool DB, class Get>
-__device__ __forceinline__ M3 around(const double2 *u, size_t ia, const FxM &F, size_t ib, const Get &get)
+__device__ __forceinline__ M3 around(const Lat &L, const double2 *u, size_t ia, const FxM &F, size_t ib, const Get &get)
 {
     const FxM A = load_fx(u, ia), B = load_fx(u, ib);
     if (A.ok() && B.ok() && F.ok()) return product<DA, DB>(A, F, B);
     M3 r = get();
-    product_f64(DA, DB, u, ia, ib, r);
+    product_f64(DA, DB, u, L.V, ia, ib, r);
     return r;
 }
 
@@ -352,13 +354,13 @@ template <class Get>
 __device__ __forceinline__ M3 stap_up(const Lat &L, const double2 *u, int mu, int nu, const int (&x)[4], const Get &get)
 {
     const size_t o = (size_t)nu * L.V;
-    return around<false, true>(u, o + site_index(L, x), to_fx(get()), o + at(L, x, mu, 1), get);
+    return around<false, true>(L, u, o + site_index(L, x), to_fx(get()), o + at(L, x, mu, 1), get);
 }
 template <class Get>
 __device__ __forceinline__ M3 stap_down(const Lat &L, const double2 *u, int mu, int nu, const int (&x)[4], const Get &get)
 {
     const size_t o = (size_t)nu * L.V;
-    return around<true, false>(u, o + at(L, x, nu, -1), to_fx(get()), o + at(L, x, nu, -1, mu, 1), get);
+    return around<true, false>(L, u, o + at(L, x, nu, -1), to_fx(get()), o + at(L, x, nu, -1, mu, 1), get);
 }
 
 struct Coef {
@@ -389,9 +391,9 @@ __global__ void __launch_bounds__(128) k_stap3(Lat L, const double2 *u, int mu, 
     coords(L, i, x);
     const size_t m = (size_t)mu * L.V, o = (size_t)nu * L.V;
     const size_t iu = m + at(L, x, nu, 1), id = m + at(L, x, nu, -1);
-    M3 up = around<false, true>(u, o + site_index(L, x), load_fx(u, iu), o + at(L, x, mu, 1), [&] { return load_link(u, iu); });
-    const M3 dn = around<true, false>(u, o + at(L, x, nu, -1), load_fx(u, id), o + at(L, x, nu, -1, mu, 1),
-                                      [&] { return load_link(u, id); });
+    M3 up = around<false, true>(L, u, o + site_index(L, x), load_fx(u, iu), o + at(L, x, mu, 1), [&] { return load_link(u, L.V, iu); });
+    const M3 dn = around<true, false>(L, u, o + at(L, x, nu, -1), load_fx(u, id), o + at(L, x, nu, -1, mu, 1),
+                                      [&] { return load_link(u, L.V, id); });
     if (td) store(td, (size_t)n * L.V + i, dn);
     else axpy(up, 1.0, dn);
     store(t, (size_t)n * L.V + i, up);
@@ -434,7 +436,7 @@ __global__ void __launch_bounds__(128) k_stap7(Lat L, const double2 *u, int mu, 
     int x[4];
     coords(L, i, x);
     M3 acc = zero();
-    axpy(acc, c.c1, load_link(u, (size_t)mu * L.V + i));
+    axpy(acc, c.c1, load_link(u, L.V, (size_t)mu * L.V + i));
 #pragma unroll 1
     for (int n = 0; n < 3; n++) {
         const int rho = n + (n >= mu);
@@ -502,38 +504,40 @@ __device__ __forceinline__ double fro2(const M3 &A)
 }
 
 // a matrix as a link of the second level (fixed point, in blocks)
-__device__ __forceinline__ void store_link(double2 *f, size_t i, const M3 &m)
+__device__ __forceinline__ void store_link(double2 *f, uint32_t V, size_t i, const M3 &m)
 {
     double d[18];
     uint32_t w[36];
+    uint64_t rest;
 #pragma unroll
     for (int k = 0; k < 9; k++) {
         d[2 * k] = m.a[k].x;
         d[2 * k + 1] = m.a[k].y;
     }
-    fx_encode_link(d, w);
+    fx_encode_link(d, w, rest);
+    const_cast<uint64_t *>(rests(f, V))[i] = rest;
     uint4 *p = reinterpret_cast<uint4 *>(const_cast<double2 *>(slot(f, i)));
 #pragma unroll
     for (int k = 0; k < 9; k++) p[32 * k] = make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
 }
 
 // the caller's thin links (records) as links of the first level
-__global__ void __launch_bounds__(128) k_take_links(const double2 *thin, double2 *u, uint64_t n)
+__global__ void __launch_bounds__(128) k_take_links(const double2 *thin, double2 *u, uint32_t V)
 {
     const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    if (t >= n) return;
+    if (t >= 4ull * V) return;
     M3 m;
 #pragma unroll
     for (int k = 0; k < 9; k++) m.a[k] = thin[t * 9 + k];
-    store_link(u, t, m);
+    store_link(u, V, t, m);
 }
 
 // W = unitary polar factor of V (scaled Newton iteration); a singular or non-converging
 // matrix raises the device error flag
-__global__ void __launch_bounds__(128) k_project_u3(const double2 *v, double2 *w, uint64_t n, DevStatus *status)
+__global__ void __launch_bounds__(128) k_project_u3(const double2 *v, double2 *w, uint32_t V, DevStatus *status)
 {
     const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    if (t >= n) return;
+    if (t >= 4ull * V) return;
     M3 X = load(v, t);
     bool ok = false, scaled = true;
     for (int it = 0; it < 30; it++) {
@@ -576,7 +580,7 @@ __global__ void __launch_bounds__(128) k_project_u3(const double2 *v, double2 *w
             break;
         }
     }
-    store_link(w, t, X);
+    store_link(w, V, t, X);
     if (!ok && status) {
         status->where = 2; // link projection
         atomicExch(&status->error, (int)HISQ_EDEVICE);
@@ -592,7 +596,7 @@ __global__ void __launch_bounds__(128) k_naik(Lat L, const double2 *w, double2 *
     int x[4];
     coords(L, i, x);
     const size_t m = (size_t)mu * L.V, j = m + at(L, x, mu, 1);
-    const M3 r = around<false, false>(w, m + i, load_fx(w, j), m + at(L, x, mu, 1, mu, 1), [&] { return load_link(w, j); });
+    const M3 r = around<false, false>(L, w, m + i, load_fx(w, j), m + at(L, x, mu, 1, mu, 1), [&] { return load_link(w, L.V, j); });
     M3 o = zero();
     axpy(o, cn, r);
     store<true>(out, (size_t)mu * L.V + i, o);
@@ -617,7 +621,7 @@ extern "C" int hisq_smear_links(const int dims[4], const double *thin, double *f
     if (V > (1ull << 31)) return HISQ_EINVAL;
     L.V = (uint32_t)V;
     L.Vh = (uint32_t)(V / 2);
-    const size_t bytes = 4 * V * 9 * sizeof(double2);
+    const size_t bytes = 4 * V * 9 * sizeof(double2), fx_bytes = bytes + 4 * V * kFxRestBytes;
     cudaStream_t st = (cudaStream_t)stream;
     double2 *u = nullptr, *v = nullptr, *w = nullptr, *x = nullptr, *nk = nullptr;
     DevStatus *status = nullptr;
@@ -625,8 +629,8 @@ extern "C" int hisq_smear_links(const int dims[4], const double *thin, double *f
         for (void *p : {(void *)u, (void *)v, (void *)w, (void *)x, (void *)nk, (void *)status})
             if (p) cudaFree(p);
     };
-    bool ok = cudaMalloc((void **)&u, bytes) == cudaSuccess && cudaMalloc((void **)&v, bytes) == cudaSuccess &&
-              cudaMalloc((void **)&w, bytes) == cudaSuccess && cudaMalloc((void **)&status, sizeof(DevStatus)) == cudaSuccess;
+    bool ok = cudaMalloc((void **)&u, fx_bytes) == cudaSuccess && cudaMalloc((void **)&v, bytes) == cudaSuccess &&
+              cudaMalloc((void **)&w, fx_bytes) == cudaSuccess && cudaMalloc((void **)&status, sizeof(DevStatus)) == cudaSuccess;
     if (ok && !links_on_device) ok = cudaMalloc((void **)&x, bytes) == cudaSuccess && cudaMalloc((void **)&nk, bytes) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -646,9 +650,9 @@ extern "C" int hisq_smear_links(const int dims[4], const double *thin, double *f
     if (e == cudaSuccess) {
         // scratch of a level (three matrices per site each): fields that hold nothing yet or no
         // longer, so no memory beyond the links, the two levels and the results is needed
-        smear::k_take_links<<<nb4, 128, 0, st>>>(src, u, 4 * V);
+        smear::k_take_links<<<nb4, 128, 0, st>>>(src, u, L.V);
         smear::smear_level<false>(L, u, v, w, nullptr, xo, smear::Coef{1.0 / 8, 1.0 / 16, 1.0 / 64, 1.0 / 384, 0.0}, st);
-        smear::k_project_u3<<<nb4, 128, 0, st>>>(v, w, 4 * V, status);
+        smear::k_project_u3<<<nb4, 128, 0, st>>>(v, w, L.V, status);
         smear::smear_level<true>(L, w, xo, u, v, no, smear::Coef{1.0, 1.0 / 16, 1.0 / 64, 1.0 / 384, -1.0 / 8}, st);
         smear::k_naik<<<dim3(nb, 4), 128, 0, st>>>(L, w, no, -1.0 / 24 + eps_naik / 8);
         e = cudaGetLastError();
