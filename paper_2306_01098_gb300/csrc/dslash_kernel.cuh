@@ -221,35 +221,77 @@ struct HopPipe {
 };
 
 // ---------------------------------------------------------------- FP64 sites in fixed point
-// the hops q2 in [q0, q1) of site s in FP64, one at a time: sites that hold what the fixed-point
-// format cannot (infinities, NaN, extreme magnitudes)
-static __device__ __noinline__ void fx_site_f64(const DslashArgs &a, const Geom &g, const char *links, size_t slot_bytes,
-                                                const char *in, uint32_t s, int q0, int q1, double (&out)[6])
+// out += hop (mu, type, back) of D in at site s in FP64; the link as doubles, - U^+ v turned into U v for the same
+// multiply-adds
+static __device__ __forceinline__ void fx_hop_f64(const DslashArgs &a, const Geom &g, const char *links, size_t slot_bytes,
+                                                  const char *in, uint32_t s, int mu, int type, bool back,
+                                                  Prec<HISQ_F64>::Acc &out)
 {
-    const Site c = site_coords(g, s, a.p);
-    for (int i = 0; i < 6; i++) out[i] = 0.0;
+    const uint32_t sn = neighbour_any(g, site_coords(g, s, a.p), s, mu, back ? (type ? -3 : -1) : (type ? 3 : 1));
+    const uint32_t sl = back ? sn : s;
+    const char *slot = links + (size_t)(((back ? 1 - a.p : a.p) * 2 + type) * 4 + mu) * slot_bytes;
+    uint32_t w[36];
+    load_link_words<144>(slot, sl, w);
+    Prec<HISQ_F64>::Link U;
+    Prec<HISQ_F64>::Vec v;
+    fx_decode_link(w, reinterpret_cast<const uint64_t *>(slot + (size_t)g.VhPad * 144)[sl], U.v);
+    Prec<HISQ_F64>::load(in, sn, v);
+    if (back) {
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+#pragma unroll
+            for (int j = 0; j < i; j++)
+#pragma unroll
+                for (int k = 0; k < 2; k++) {
+                    const double x = U.v[2 * (3 * i + j) + k];
+                    U.v[2 * (3 * i + j) + k] = U.v[2 * (3 * j + i) + k];
+                    U.v[2 * (3 * j + i) + k] = x;
+                }
+#pragma unroll
+        for (int i = 0; i < 9; i++) U.v[2 * i] = -U.v[2 * i];
+    }
+    Prec<HISQ_F64>::hop<false, false>(out, U, v);
+}
+
+// D in in FP64 at the sites of the warp's lanes in m (each lane's own s and in; all lanes call), for sites that
+// hold what the fixed-point format cannot (infinities, NaN, extreme magnitudes) or whose components it does
+// not hold to FP64's precision for certain.  Few sites (the rule): two at a time, a lane for every hop; a lane alone
+// with its site's 16 hops keeps its block for 50 to 85 us (a fifth of the warps with such a site on 32^3 x 8:
+// 163 us that way, 88 us so, 66 us without).  More than half of them (a vector of one colour): every lane its
+// own site, as its links are then read as whole lines (214 us so, 364 us two at a time).
+static __device__ __noinline__ void fx_sites_f64(const DslashArgs &a, const Geom &g, const char *links, size_t slot_bytes,
+                                                 const char *in, uint32_t s, uint32_t m, double (&out)[6])
+{
+    const int lane = threadIdx.x & 31;
+    Prec<HISQ_F64>::Acc acc;
+    if (__popc(m) > 16) {
+        if (!(m >> lane & 1u)) return;
+        Prec<HISQ_F64>::zero(acc);
 #pragma unroll 1
-    for (int q = 2 * q0; q < 2 * q1; q++) {
-        const int mu = q >> 2, type = (q >> 1) & 1, k = type ? 3 : 1;
-        const bool back = q & 1;
-        bool wrap;
-        const uint32_t sn = neighbour(g, c, s, mu, back ? -k : k, wrap);
-        const int lp = back ? 1 - a.p : a.p;
-        uint32_t w[36];
-        const char *slot = links + (size_t)((lp * 2 + type) * 4 + mu) * slot_bytes;
-        load_link_words<144>(slot, back ? sn : s, w);
-        const uint64_t rest = reinterpret_cast<const uint64_t *>(slot + (size_t)g.VhPad * 144)[back ? sn : s];
-        Prec<HISQ_F64>::Link U;
-        Prec<HISQ_F64>::Vec v;
-        Prec<HISQ_F64>::Acc acc;
-        fx_decode_link(w, rest, U.v);
+        for (int q = 0; q < 16; q++) fx_hop_f64(a, g, links, slot_bytes, in, s, q >> 2, (q >> 1) & 1, q & 1, acc);
 #pragma unroll
-        for (int i = 0; i < 6; i++) acc.v[i] = out[i];
-        Prec<HISQ_F64>::load(in, sn, v);
-        if (back) Prec<HISQ_F64>::hop<true, true>(acc, U, v);
-        else Prec<HISQ_F64>::hop<false, false>(acc, U, v);
+        for (int k = 0; k < 6; k++) out[k] = acc.v[k];
+        return;
+    }
+#pragma unroll 1
+    while (m) {
+        const int l0 = __ffs((int)m) - 1;
+        m &= m - 1;
+        const int l1 = m ? __ffs((int)m) - 1 : l0;
+        m &= m - 1;
+        const int src = lane < 16 ? l0 : l1;
+        const uint32_t ss = __shfl_sync(0xffffffffu, s, src);
+        const char *si = reinterpret_cast<const char *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(in), src));
+        Prec<HISQ_F64>::zero(acc);
+        fx_hop_f64(a, g, links, slot_bytes, si, ss, (lane >> 2) & 3, (lane >> 1) & 1, lane & 1, acc);
 #pragma unroll
-        for (int i = 0; i < 6; i++) out[i] = acc.v[i];
+        for (int k = 0; k < 6; k++) {
+#pragma unroll
+            for (int off = 8; off > 0; off >>= 1) acc.v[k] += __shfl_xor_sync(0xffffffffu, acc.v[k], off);
+            const double x0 = __shfl_sync(0xffffffffu, acc.v[k], 0), x1 = __shfl_sync(0xffffffffu, acc.v[k], 16);
+            if (lane == l0) out[k] = x0;
+            else if (lane == l1) out[k] = x1;
+        }
     }
 }
 
@@ -260,8 +302,6 @@ __device__ __forceinline__ void fx_site(const DslashArgs &a, const Geom &g, cons
                                         const char *in, uint32_t s, bool live, int part,
                                         Prec<HISQ_F64>::Acc (&out)[NR])
 {
-    constexpr int NQ = 8 / DS;
-    const int q0 = part * NQ;
     FxAcc acc[NR];
 #pragma unroll
     for (int r = 0; r < NR; r++) fx_zero(acc[r]);
@@ -276,37 +316,35 @@ __device__ __forceinline__ void fx_site(const DslashArgs &a, const Geom &g, cons
             for (int h = 0; h < 4; h++) {
                 uint32_t w[36];
                 pipe.link(h, w);
-                const uint32_t code = fx_take_code(w);
+                uint32_t f;
+                const uint32_t code = fx_take_code(w, f);
 #pragma unroll
                 for (int r = 0; r < NR; r++) {
                     uint32_t x[12];
                     pipe.vec(h, r, x);
-                    if (h & 1) fx_hop<true>(acc[r], w, code, x);
-                    else fx_hop<false>(acc[r], w, code, x);
+                    if (h == 0) fx_hop<false, true>(acc[r], w, code, f, x);
+                    else if (h == 1) fx_hop<true, true>(acc[r], w, code, f, x);
+                    else if (h == 2) fx_hop<false, false>(acc[r], w, code, f, x);
+                    else fx_hop<true, false>(acc[r], w, code, f, x);
                 }
                 pipe.next(m, h);
             }
     }
-    bool bad = false;
+    bool left = false;
 #pragma unroll
     for (int r = 0; r < NR; r++) {
         if constexpr (DS > 1) fx_combine<DS>(acc[r]);
 #pragma unroll
         for (int k = 0; k < 6; k++) out[r].v[k] = fx_value(acc[r], k);
-        bad |= acc[r].bad;
+        acc[r].bad = fx_left(acc[r]);
+        left |= acc[r].bad;
     }
-    if (__any_sync(0xffffffffu, bad)) {
+    if (__any_sync(0xffffffffu, left)) {
 #pragma unroll
         for (int r = 0; r < NR; r++) {
-            double o[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-            if (live && acc[r].bad)
-                fx_site_f64(a, g, links, slot_bytes, in + (size_t)r * a.rhs_bytes, s, q0, q0 + NQ, o);
-#pragma unroll
-            for (int k = 0; k < 6; k++) {
-#pragma unroll
-                for (int off = 16; off >= 32 / DS; off >>= 1) o[k] += __shfl_xor_sync(0xffffffffu, o[k], off);
-                if (acc[r].bad) out[r].v[k] = o[k];
-            }
+            // (the first of a site's threads goes on with the result)
+            const uint32_t m = __ballot_sync(0xffffffffu, acc[r].bad && part == 0);
+            if (m) fx_sites_f64(a, g, links, slot_bytes, in + (size_t)r * a.rhs_bytes, s, m, out[r].v);
         }
     }
 }

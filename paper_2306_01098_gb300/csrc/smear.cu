@@ -211,7 +211,8 @@ __device__ __forceinline__ FxM load_fx(const double2 *f, size_t i)
     uint32_t w[36];
     link_words(f, i, w);
     FxM r;
-    r.code = fx_take_code(w);
+    uint32_t rows;
+    r.code = fx_take_code(w, rows);
 #pragma unroll
     for (int k = 0; k < 18; k++) {
         r.l[k] = (int32_t)w[2 * k];

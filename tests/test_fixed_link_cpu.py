@@ -19,10 +19,12 @@ int main()
         uint64_t rest;
         hisq::fx_encode_link(d, w, rest);
         hisq::fx_decode_link(w, rest, back);
-        const int32_t code = (int32_t)hisq::fx_take_code(w);
+        uint32_t f;
+        const int32_t code = (int32_t)hisq::fx_take_code(w, f);
         fwrite(back, 8, 18, stdout);
         fwrite(w, 4, 36, stdout);
         fwrite(&code, 4, 1, stdout);
+        fwrite(&f, 4, 1, stdout);
     }
 }
 """
@@ -42,7 +44,7 @@ def roundtrip(tmp_path_factory):
     def run(links):
         out = subprocess.run([str(exe)], input=np.ascontiguousarray(links, dtype=np.float64).tobytes(), check=True,
                              capture_output=True).stdout
-        rec = np.frombuffer(out, dtype=[("back", "<f8", 18), ("w", "<i4", (18, 2)), ("code", "<i4")])
+        rec = np.frombuffer(out, dtype=[("back", "<f8", 18), ("w", "<i4", (18, 2)), ("code", "<i4"), ("f", "<i4")])
         assert len(rec) == len(links)
         return rec
 
@@ -95,3 +97,17 @@ def test_doubles_come_back(roundtrip, kind):
             cut = num * 2 ** -unit // den if unit < 0 else num // (den * 2 ** unit)
             assert abs(int(x[i, k])) == cut and (cut == 0 or (int(x[i, k]) < 0) == (d[i, k] < 0))
     assert (np.abs(rec["w"][fx][:, :, 1]) <= 2 ** 28).all()
+
+
+@pytest.mark.parametrize("kind", ["plain", "sparse", "spread", "binade edges", "named"])
+def test_balance_of_a_link(roundtrip, kind):
+    # f 2^e is no more than any row or column sum of |reals|, and as large as that allows (up to the cut)
+    d = _links(kind)
+    rec = roundtrip(d)
+    fx = (rec["code"] != 0xfff) & (rec["code"] != 0)
+    a = np.abs(d).reshape(-1, 3, 3, 2).sum(-1)
+    least = np.minimum(a.sum(1).min(1), a.sum(2).min(1))[fx] / np.exp2(rec["code"][fx] - 1023.0)
+    f = rec["f"][fx]
+    assert (f <= least).all() and (f >= np.minimum(3, np.floor(least - 1e-7))).all()
+    unitary = np.linalg.qr(np.random.default_rng(3).normal(size=(200, 3, 3, 2)).view(np.complex128)[..., 0])[0] * 0.3
+    assert (roundtrip(unitary.reshape(200, 9).view(np.float64))["f"] >= 1).all()
