@@ -271,14 +271,59 @@ __device__ __forceinline__ void fold(FxRow &r)
     }
 }
 
-// op(A) F op(B) with op the adjoint where DA, DB say so, for codes in range.  Row by row: row i of
-// op(A) F, brought back to two limbs (its sums of six products stay below 2^90.6, 31 bits off leave 2^59.6;
-// the exponent is then cA + cF - 1019), times op(B).
-template <bool DA, bool DB>
-__device__ __forceinline__ M3 product(const FxM &A, const FxM &F, const FxM &B)
+// 1-norm of complex entry q in units of 2^-13 of 2^e, cut, at most 2^15
+__device__ __forceinline__ uint32_t norm1(const FxM &m, int q)
 {
-    M3 out;
-    const uint32_t E = A.code + F.code - 1019u + B.code;
+    const int32_t r = m.h[2 * q], i = m.h[2 * q + 1];
+    return ((uint32_t)(r ^ (r >> 31)) + (uint32_t)(i ^ (i >> 31))) >> 14;
+}
+// What enters the entries of row i of op(A) F op(B): S_ik = sum_jl |A_ij| |F_jl| |B_lk| in 1-norms of the entries;
+// the least of a row in units of 2^-22 of 2^(eA + eF + eB)
+template <bool DA, bool DB>
+__device__ __forceinline__ void least_sums(const FxM &A, const FxM &F, const FxM &B, uint32_t (&m)[3])
+{
+    uint32_t g[9];
+#pragma unroll
+    for (int j = 0; j < 3; j++)
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            uint32_t x = 0;
+#pragma unroll
+            for (int l = 0; l < 3; l++) x += norm1(F, 3 * j + l) * norm1(B, DB ? 3 * k + l : 3 * l + k);
+            g[3 * j + k] = x >> 17;
+        }
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        m[i] = 0xffffffffu;
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            uint32_t x = 0;
+#pragma unroll
+            for (int j = 0; j < 3; j++) x += norm1(A, DA ? 3 * j + i : 3 * i + j) * g[3 * j + k];
+            m[i] = min(m[i], x);
+        }
+    }
+}
+
+// op(A) F op(B) with op the adjoint where DA, DB say so, for codes in range; false if the result may be less
+// precise than FP64's.  Row by row: row i of op(A) F, brought back to two limbs (its sums of six products
+// stay below 2^90.6; the shift sh <= 31 leaves its largest entry 59 or 60 bits), times op(B).
+// Error of an entry's real or imaginary part, at most, in units of 2^-56 of 2^(eA + eF + eB): six products of the
+// first kind, 1.75 each (fixed.cuh), a row cut to units of 2^(sh - 30) (and one more where a limb was negated),
+// all times twelve, then 2^(sh - 27) for each l l' of the second and the cut of B: 126 + 10.5 2^(sh - 27).
+// FP64 multiply-adds err by up to 12 2^-53 S.  Both worked out in exact arithmetic for 8,600 entries of products of
+// links and staples at eps 0.03 to 1 (sh - 27 mostly 2): the fixed-point ones err less, 0.38 2^-53 S against 0.40
+// (rms) and 1.1 against 1.9 (largest), from S = 0.75 on (0.48 against 0.37 below that; 0.10 against 0.25 from 10
+// on).  So an entry needs S >= 0.5 + 2^(sh - 31).  Products that have less at eps 0.5: none, at 0.3 4e-5
+// (second level; its links are smoother), at 0.2 0.4 %, at 0.1 28 %, closer to unity nearly all: 24^3 x 8 in
+// 6.9, 7.2, 8.1, 18.1 ms, 13.7 ms at eps 0.001 (6.7 whatever the links without looking).
+template <bool DA, bool DB>
+__device__ __forceinline__ bool product(const FxM &A, const FxM &F, const FxM &B, M3 &out)
+{
+    uint32_t least[3];
+    least_sums<DA, DB>(A, F, B, least);
+    bool ok = min(least[0], min(least[1], least[2])) >= 2097152u;
+    if (!ok) return false;
 #pragma unroll
     for (int i = 0; i < 3; i++) {
         FxRow r = {};
@@ -298,12 +343,18 @@ __device__ __forceinline__ M3 product(const FxM &A, const FxM &F, const FxM &B)
             }
         }
         fold(r);
+        uint32_t top = 0;
+#pragma unroll
+        for (int k = 0; k < 6; k++) top |= (uint32_t)(r.H[k] >> 32) ^ (uint32_t)(r.H[k] >> 63);
+        const uint32_t sh = 36u - (uint32_t)__clz((int)top); // 4 .. 31
+        const uint32_t E = A.code + F.code + B.code - 1050u + sh;
+        ok = ok && least[i] >= 2097152u + ((1u << sh) >> 9);
         int32_t ph[6], pl[6];
 #pragma unroll
         for (int k = 0; k < 6; k++) {
-            const int64_t x = (int64_t)((uint64_t)r.H[k] << 1 | (uint32_t)r.M[k] >> 31);
-            pl[k] = (int32_t)(uint32_t)x;
-            ph[k] = (int32_t)(x >> 32) + (int32_t)((uint32_t)pl[k] >> 31);
+            const uint32_t lo = (uint32_t)r.H[k];
+            pl[k] = (int32_t)__funnelshift_r((uint32_t)r.M[k], lo, sh);
+            ph[k] = (int32_t)__funnelshift_r(lo, (uint32_t)(r.H[k] >> 32), sh) + (int32_t)((uint32_t)pl[k] >> 31);
         }
         FxRow o = {};
 #pragma unroll
@@ -326,10 +377,10 @@ __device__ __forceinline__ M3 product(const FxM &A, const FxM &F, const FxM &B)
             out.a[3 * i + k] = make_double2(fx_value(o.H[2 * k], (uint32_t)o.M[2 * k], E),
                                             fx_value(o.H[2 * k + 1], (uint32_t)o.M[2 * k + 1], E));
     }
-    return out;
+    return ok;
 }
 
-// the same in FP64, for matrices that the fixed-point range leaves out
+// the same in FP64, for matrices that the fixed-point range or precision leaves out
 static __device__ __noinline__ void product_f64(bool da, bool db, const double2 *u, uint32_t V, size_t ia, size_t ib, M3 &F)
 {
     const M3 A = load_link(u, V, ia), B = load_link(u, V, ib);
@@ -342,8 +393,9 @@ template <bool DA, bool DB, class Get>
 __device__ __forceinline__ M3 around(const Lat &L, const double2 *u, size_t ia, const FxM &F, size_t ib, const Get &get)
 {
     const FxM A = load_fx(u, ia), B = load_fx(u, ib);
-    if (A.ok() && B.ok() && F.ok()) return product<DA, DB>(A, F, B);
-    M3 r = get();
+    M3 r;
+    if (A.ok() && B.ok() && F.ok() && product<DA, DB>(A, F, B, r)) return r;
+    r = get();
     product_f64(DA, DB, u, L.V, ia, ib, r);
     return r;
 }
@@ -382,7 +434,8 @@ struct Coef {
 // issue at eight warps an SM (the operands of a product fill the registers).  One thread per (site,
 // detour) in launches 1 and 2, one per site in 3, consecutive sites in consecutive lanes.
 // 24^3 x 8, the whole call with projection and Naik links: 76.0 ms with every path multiplied out, 12.4
-// with stored staples in FP64, 7.6 with these products, 6.6 with the projection of now.
+// with stored staples in FP64, 7.6 with these products, 6.7 with the projection of now, 7.0 with the look at what
+// enters each entry (product).
 __global__ void __launch_bounds__(128) k_stap3(Lat L, const double2 *u, int mu, double2 *t, double2 *td)
 {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
