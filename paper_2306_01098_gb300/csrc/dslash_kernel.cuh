@@ -752,9 +752,12 @@ static cudaError_t launch_one(const DslashArgs &a0, cudaStream_t st)
     if (bs != 64 && bs != 128 && bs != 256) return cudaErrorInvalidValue;
     a.bs = bs;
     const size_t smem = (size_t)bs * PipeShape<PL, PV, NREAL, NR, DS>::bytes;
-    if (smem > 32 * 1024) { // (48 KB with the static part) a per-device attribute of the function
+    if (smem > 32 * 1024) { // (48 KB with the static part)
+        // The attribute belongs to the function and device, not to this launch: always the most that any block
+        // size takes, so that no thread lowers it between another's setting and its launch.
         cudaError_t e = cudaFuncSetAttribute(k_dslash<PL, PV, NREAL, NR, EPI, DS, BATCH, RG, WG>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kDslashMaxBlock * PipeShape<PL, PV, NREAL, NR, DS>::bytes);
         if (e != cudaSuccess) return e;
     }
     static int occ[3] = {-1, -1, -1}; // resident blocks per SM of this instantiation, per block size
