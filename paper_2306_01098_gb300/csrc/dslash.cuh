@@ -18,7 +18,7 @@ struct DslashArgs {
     const char *in;        // input field, parity 1-p, right-hand side 0
     char *out;             // output field, parity p
     size_t rhs_bytes;      // bytes between right-hand sides
-    int out64;             // out is canonical FP64, [nrhs][Vh] 48-byte records on 16-byte boundaries
+    int out64;             // plain Dslash: out is canonical FP64, [nrhs][Vh] 48-byte records on 16-byte boundaries
     int nrhs;
     const Scalars *skip;   // if set: return at once when no right-hand side is active
     // normal-operator epilogue: out = m4 * pv - D in, <pv, out> reduced; with the CG

@@ -30,7 +30,9 @@
 // Optional epilogue (normal operator, Sec. 3.2 applyMdaggM):
 //   EPI = 1: out = m4 * p - D in,   and <p, out> reduced in FP64 per right-hand side;
 //   EPI = 2: the same and also |r|^2, <r, out> and <out, out> (four values per right-hand
-//            side, from which the CG finishing step gets alpha and the next |r|^2).
+//            side, from which the CG finishing step gets alpha and the next |r|^2);
+//   EPI = 3: out = m4 * p - D in as canonical FP64, no dot products (hisq_mdagm; a kernel of its own, as
+//            its store cost the solvers' EPI = 1 up to 2 %: two sides, 16-bit links, 32^3 x 8, 15.6 against 15.3 ms).
 // Batches: one launch over the lattices of a batch, each with its own geometry and links
 // (one right-hand side per lattice); a block finds its lattice in the batch table.
 #pragma once
@@ -46,6 +48,14 @@ namespace hisq {
 
 // dot products per right-hand side reduced by an epilogue
 template <int EPI> struct EpiDots { static constexpr int n = EPI == 2 ? 4 : 1; };
+
+// the output is canonical FP64: EPI = 3, or a plain Dslash of one lattice that says so
+template <int EPI, bool PLAIN64>
+__device__ __forceinline__ bool canonical_out(const DslashArgs &a)
+{
+    if constexpr (EPI == 3) return true;
+    else return EPI == 0 && PLAIN64 && a.out64;
+}
 
 // |v|^2 and |o|^2 of FP32 records in float arithmetic, returned as floats
 __device__ __forceinline__ float vec_norm2f(const FloatArith::Vec &v)
@@ -104,7 +114,11 @@ __device__ __forceinline__ double acc_norm2(const typename T::Acc &o)
 }
 
 // bytes between the right-hand sides of the output
-__device__ __forceinline__ size_t out_stride(const DslashArgs &a) { return a.out64 ? (size_t)a.g.Vh * 48 : a.rhs_bytes; }
+template <int EPI, bool PLAIN64>
+__device__ __forceinline__ size_t out_stride(const DslashArgs &a)
+{
+    return canonical_out<EPI, PLAIN64>(a) ? (size_t)a.g.Vh * 48 : a.rhs_bytes;
+}
 
 // vector load: the read-only path, or (COH) ordinary loads for vectors that other blocks of
 // the same launch write between grid barriers
@@ -362,9 +376,10 @@ __device__ __forceinline__ void fx_site(const DslashArgs &a, const Geom &g, cons
 // are the same addresses in the same instruction (one request), so a link is fetched once
 // for all NR RG right-hand sides with 1/RG of the accumulators per thread.
 // LL1: links allocate in L1 (right-hand-side groups of one block read the same links).
-// PIPE: the hops' operands come through shared memory (pipe_hops); else through registers.
+// PIPE: the hops' operands come through shared memory (HopPipe); else through registers.
+// PLAIN64: a plain Dslash may write canonical FP64 (DslashArgs::out64).
 template <int PL, int PV, int NREAL, int NR, int EPI, int DS, bool COH = false, bool PF = false, int RG = 1,
-          class DT = double, bool LL1 = false, bool PIPE = false>
+          class DT = double, bool LL1 = false, bool PIPE = false, bool PLAIN64 = false>
 __device__ __forceinline__ void dslash_item(const DslashArgs &a, const Geom &g, const char *links, size_t slot_bytes,
                                             std::conditional_t<std::is_same<DT, FF>::value, float, double> sc0,
                                             std::conditional_t<std::is_same<DT, FF>::value, float, double> sc1,
@@ -400,7 +415,7 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const Geom &g, 
     if constexpr (RG > 1) {
         const size_t goff = (size_t)(gt % RG) * NR * a.rhs_bytes;
         in += goff;
-        outp += COH ? goff : (size_t)(gt % RG) * NR * out_stride(a);
+        outp += (size_t)(gt % RG) * NR * out_stride<EPI, PLAIN64>(a);
         if (pvp) pvp += goff;
         if (rvp) rvp += goff;
         if (m4r) m4r += (gt % RG) * NR;
@@ -568,10 +583,10 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const Geom &g, 
                 vec_load<T, COH>(pvp + (size_t)r * a.rhs_bytes, s - ebase, pv);
                 if constexpr (FFD) {
                     T::mdagm_epilogue(out[r], m4r ? a.m4f + (float)m4r[r] : a.m4f, pv);
-                    ff_add(dots[r * ND], T::dotf(pv, out[r]));
+                    if constexpr (EPI != 3) ff_add(dots[r * ND], T::dotf(pv, out[r]));
                 } else {
                     T::mdagm_epilogue(out[r], a.m4 + (m4r ? m4r[r] : 0.0), pv);
-                    dots[r * ND] += T::dot(pv, out[r]);
+                    if constexpr (EPI != 3) dots[r * ND] += T::dot(pv, out[r]);
                 }
                 if constexpr (EPI == 2) {
                     typename T::Vec rv;
@@ -587,8 +602,8 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const Geom &g, 
                     }
                 }
             }
-            if (!COH && a.out64) { // the caller's FP64 buffer, without a pass of its own
-                double2 *q = reinterpret_cast<double2 *>(outp + (size_t)r * out_stride(a) + (size_t)s * 48);
+            if (canonical_out<EPI, PLAIN64>(a)) { // the caller's FP64 buffer, without a pass of its own
+                double2 *q = reinterpret_cast<double2 *>(outp + (size_t)r * out_stride<EPI, PLAIN64>(a) + (size_t)s * 48);
 #pragma unroll
                 for (int i = 0; i < 3; i++) q[i] = make_double2(T::canon(out[r], 2 * i), T::canon(out[r], 2 * i + 1));
             } else {
@@ -608,12 +623,6 @@ __device__ __forceinline__ void block_sum_dots(D (&d)[N])
 __device__ __forceinline__ double dot_value(const FF &x) { return ff_value(x); }
 __device__ __forceinline__ double dot_value(double x) { return x; }
 
-// BATCH: the lattices of a batch in one launch (NR = 1; right-hand side k is lattice k).
-// RG: groups of right-hand sides sharing a site's threads (dslash_item).
-// WG > 1 (no epilogue, one thread per site, RG = 1): the block's threads form WG slices of
-// a.bs threads over the same sites, slice g taking the g-th of the block's WG groups of NR
-// right-hand sides; their link loads allocate in L1, so one L2 read of a link serves the
-// block's WG NR right-hand sides without the registers of WG NR accumulators per thread.
 // 256-thread blocks per SM that the registers are limited for.  Left alone the compiler moves the
 // loads of all 16 hops to the front of the site (250 registers, 8 warps an SM); the gathers want warps:
 // FP32 vectors 48 / 64 / 128 registers at 1 / 2 / 4 right-hand sides a thread (14-shift FP32 solve
@@ -625,6 +634,13 @@ constexpr int min_blocks(int pl, int pv, int nreal, int nr)
     const int less = nreal == 12 ? 1 : 0;
     return nr == 1 ? 5 - less : nr == 2 ? 4 - less : nr == 4 ? 2 : 1;
 }
+
+// BATCH: the lattices of a batch in one launch (NR = 1; right-hand side k is lattice k).
+// RG: groups of right-hand sides sharing a site's threads (dslash_item).
+// WG > 1 (no epilogue, one thread per site, RG = 1): the block's threads form WG slices of
+// a.bs threads over the same sites, slice g taking the g-th of the block's WG groups of NR
+// right-hand sides; their link loads allocate in L1, so one L2 read of a link serves the
+// block's WG NR right-hand sides without the registers of WG NR accumulators per thread.
 template <int PL, int PV, int NREAL, int NR, int EPI, int DS, bool BATCH, int RG = 1, int WG = 1>
 __global__ void __launch_bounds__(kDslashMaxBlock, min_blocks(PL, PV, NREAL, NR)) k_dslash(const DslashArgs a)
 {
@@ -717,10 +733,10 @@ __global__ void __launch_bounds__(kDslashMaxBlock, min_blocks(PL, PV, NREAL, NR)
         const auto sc0 = [&] { if constexpr (FFK) return a.scale_f[0]; else return a.scale[0]; }();
         const auto sc1 = [&] { if constexpr (FFK) return a.scale_f[1]; else return a.scale[1]; }();
         for (uint32_t item = blockIdx.x; item < a.items; item += gridDim.x)
-            dslash_item<PL, PV, NREAL, NR, EPI, DS, false, false, RG, DTK, (WG > 1), PipeShape<PL, PV, NREAL, NR, DS>::on>(
-                a, a.g, a.links, a.slot_bytes, sc0, sc1, a.in + off, a.out + (size_t)rhs0 * out_stride(a), EPI ? a.pv + off : nullptr,
+            dslash_item<PL, PV, NREAL, NR, EPI, DS, false, false, RG, DTK, (WG > 1), PipeShape<PL, PV, NREAL, NR, DS>::on, true>(
+                a, a.g, a.links, a.slot_bytes, sc0, sc1, a.in + off, a.out + (size_t)rhs0 * out_stride<EPI, true>(a), EPI ? a.pv + off : nullptr,
                 EPI == 2 ? a.rv + off : nullptr, a.shift ? a.shift + rhs0 : nullptr, item / ngroups, dots, tid);
-        if constexpr (EPI >= 1) {
+        if constexpr (EPI == 1 || EPI == 2) {
             if (a.red.partials) { // uniform over the grid
                 if constexpr (RG == 1) {
                     block_sum_dots<FFK, NR * ND>(dots);
@@ -803,8 +819,11 @@ static cudaError_t launch_nr(const DslashArgs &a, int nr, int rg, cudaStream_t s
 {
     if (a.nrhs < 1 || a.nrhs % (nr * rg)) return cudaErrorInvalidValue;
     if (a.batch) { // one right-hand side per lattice, storage order
-        if (nr != 1 || rg != 1 || a.zt || a.nrhs != a.batch_n) return cudaErrorInvalidValue;
-        return launch_one<PL, PV, NREAL, 1, EPI, DS, true>(a, st);
+        if constexpr (EPI == 3) return cudaErrorInvalidValue;
+        else {
+            if (nr != 1 || rg != 1 || a.zt || a.nrhs != a.batch_n) return cudaErrorInvalidValue;
+            return launch_one<PL, PV, NREAL, 1, EPI, DS, true>(a, st);
+        }
     }
     if (a.zt && !a.g.zt_ok) return cudaErrorInvalidValue;
     if (a.wg > 1) { // slices of a block over the same sites: plain Dslash, one thread per site
@@ -867,18 +886,20 @@ static cudaError_t launch_prec(const DslashArgs &a, int nreal, int nr, int ds, i
     return launch_ds<PL, PV, 18, EPI>(a, nr, ds, rg, st);
 }
 
-// instantiate the launcher of one link precision with one vector precision
-// (the CG epilogue, EPI = 2, exists for the vector precisions a solver iterates: not 16-bit)
+// Instantiate the launcher of one link precision with one vector precision.  Epilogues exist for the vector
+// precisions that a solver iterates (not 16-bit); EPI = 3 for those that are not canonical by themselves.
 #define HISQ_DSLASH_INSTANTIATE(PL, PV)                                                                  \
     cudaError_t dslash_launch_##PL##_##PV(int epi, const DslashArgs &a, int nreal, int nr, int ds, int rg, \
                                           cudaStream_t st)                                               \
     {                                                                                                    \
-        if (epi == 2) {                                                                                  \
-            if constexpr (PV == HISQ_F16 || PV == HISQ_BF16) return cudaErrorInvalidValue;              \
-            else return launch_prec<PL, PV, 2>(a, nreal, nr, ds, rg, st);                                 \
+        if (epi == 0) return launch_prec<PL, PV, 0>(a, nreal, nr, ds, rg, st);                           \
+        if constexpr (PV != HISQ_F16 && PV != HISQ_BF16) {                                               \
+            if (epi == 1) return launch_prec<PL, PV, 1>(a, nreal, nr, ds, rg, st);                       \
+            if (epi == 2) return launch_prec<PL, PV, 2>(a, nreal, nr, ds, rg, st);                       \
+            if constexpr (PV != HISQ_F64)                                                                \
+                if (epi == 3) return launch_prec<PL, PV, 3>(a, nreal, nr, ds, rg, st);                   \
         }                                                                                                \
-        return epi ? launch_prec<PL, PV, 1>(a, nreal, nr, ds, rg, st)                                    \
-                   : launch_prec<PL, PV, 0>(a, nreal, nr, ds, rg, st);                                   \
+        return cudaErrorInvalidValue;                                                                    \
     }
 
 }  // namespace hisq

@@ -48,11 +48,8 @@ int apply_mdagm(hisq_ctx *ctx, int prec, double m, const void *in, void *tmp, vo
     b.pv = static_cast<const char *>(in);
     b.m4 = 4.0 * m * m;
     if (red) b.red = *red;
-    if (out64) {
-        b.out = reinterpret_cast<char *>(out64);
-        b.out64 = 1;
-    }
-    e = dslash_launch(prec, pv, 1, b, L.nreal, sh, st);
+    if (out64) b.out = reinterpret_cast<char *>(out64); // (no dot products: EPI = 3)
+    e = dslash_launch(prec, pv, out64 ? 3 : 1, b, L.nreal, sh, st);
     if (e != cudaSuccess) return cuda_error(ctx, e, "dslash D_eo + epilogue");
     return HISQ_OK;
 }
