@@ -624,14 +624,29 @@ __device__ __forceinline__ double dot_value(const FF &x) { return ff_value(x); }
 __device__ __forceinline__ double dot_value(double x) { return x; }
 
 // 256-thread blocks per SM that the registers are limited for.  Left alone the compiler moves the
-// loads of all 16 hops to the front of the site (250 registers, 8 warps an SM); the gathers want warps:
-// FP32 vectors 48 / 64 / 128 registers at 1 / 2 / 4 right-hand sides a thread (14-shift FP32 solve
-// 32^3 x 8: 74 ms without limits, 63 ms with 64 / 80 / 128, 59 ms so; one block less for rebuilt third
-// rows), FP64 and float pairs 128 at one.
-constexpr int min_blocks(int pl, int pv, int nreal, int nr)
+// loads of all 16 hops to the front of the site (250 registers, 8 warps an SM); the gathers want warps, the
+// dot products want registers (limits that leave too few spill 170 to 380 bytes).  FP32 vectors, registers per
+// kernel and us per iteration of a solve on 32^3 x 8 and x 16 (uneven batch of 32 lattices: ms):
+//   no dot products     48 / 64 / 128 at 1 / 2 / 4 right-hand sides a thread (14-shift FP32 solve 32^3 x 8: 74 ms
+//                       without limits, 63 ms with 64 / 80 / 128, 59 ms so)
+//   EPI = 1, one side   16-bit links 64: 56.5, 84.1 (48: 59.8, 89.5; no limit 56.3, 86.3, but 422 for 8 groups of one
+//                       on x 16, where 64 take 368); FP32 links no limit: 76.1, 124 (64: 76.9, 127; 48: 79.8, 135)
+//   EPI = 1, two, four  64 / 128: FP32 links, two 86.8, 147 (80: 97.7, 155), four 123, 199 (no limit 131, 211)
+//   EPI = 2, one, two   no limit: 16-bit links 54.3, 82.7 and 80.3, 123 (48: 62.0, 96.2; 64: 88.8, 128)
+//   EPI = 2, four       128: 16-bit links, 8 sides 210, 310 (no limit 211, 337)
+//   batch               FP32 links no limit: 57.3, EPI = 2 62.4 (48: 59.0, 71.3); 16-bit links 64: 42.6, 48.9 (48: 47.6,
+//                       55.6); the kernel without dot products alike, as its time chooses the threads per site of all
+// One block less for rebuilt third rows (their EPI = 1 too: FP32 links 64.5, 95.9, no limit 66.1, 95.5).  FP64 and
+// float pairs: 128 at one side (float pairs, four sides in groups of one: 437, 802, no limit 520, 962; FP64 batch 133
+// ms, no limit 150).
+constexpr int min_blocks(int pl, int pv, int nreal, int nr, int epi, bool batch, int rg)
 {
     if (pv == HISQ_F64 || pv == HISQ_F64X) return nr == 1 && !(pl == HISQ_F64 && nreal == 12) ? 2 : 1;
     const int less = nreal == 12 ? 1 : 0;
+    if (batch) return pl == HISQ_F32 ? 1 : 4 - less;
+    if (epi == 2 && nr <= 2) return 1;
+    if (epi == 1 && nr <= 2 && rg > 1) return 1;
+    if (epi == 1 && nr == 1 && nreal == 18) return pl == HISQ_F32 ? 1 : 4;
     return nr == 1 ? 5 - less : nr == 2 ? 4 - less : nr == 4 ? 2 : 1;
 }
 
@@ -642,7 +657,7 @@ constexpr int min_blocks(int pl, int pv, int nreal, int nr)
 // right-hand sides; their link loads allocate in L1, so one L2 read of a link serves the
 // block's WG NR right-hand sides without the registers of WG NR accumulators per thread.
 template <int PL, int PV, int NREAL, int NR, int EPI, int DS, bool BATCH, int RG = 1, int WG = 1>
-__global__ void __launch_bounds__(kDslashMaxBlock, min_blocks(PL, PV, NREAL, NR)) k_dslash(const DslashArgs a)
+__global__ void __launch_bounds__(kDslashMaxBlock, min_blocks(PL, PV, NREAL, NR, EPI, BATCH, RG)) k_dslash(const DslashArgs a)
 {
     static_assert(WG == 1 || (EPI == 0 && DS == 1 && RG == 1 && !BATCH), "block slices: plain Dslash, one thread per site");
     using T = Prec<PV>;
