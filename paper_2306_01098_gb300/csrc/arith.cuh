@@ -243,13 +243,8 @@ template <> struct Prec<HISQ_F64> {
     struct Vec { double v[6]; };
     struct Acc { double v[6]; };
     static constexpr int SB = 48;
-    // chunk q of site s, and the record's words as a vector
+    // chunk q of site s
     __device__ static size_t chunk_off(uint32_t s, int q) { return (size_t)s * SB + 16 * q; }
-    __device__ static void vec_words(const uint32_t (&w)[12], Vec &v)
-    {
-#pragma unroll
-        for (int i = 0; i < 6; i++) v.v[i] = __hiloint2double((int)w[2 * i + 1], (int)w[2 * i]);
-    }
     template <int NREAL>
     __device__ static void unpack(const uint32_t *w, Link &U)
     {
@@ -433,6 +428,7 @@ struct FloatArith {
 
 template <> struct Prec<HISQ_F32> : FloatArith {
     static constexpr int SB = 24;
+    // chunk q of site s, and the record's words as a vector
     __device__ static size_t chunk_off(uint32_t s, int q) { return blocked_off<SB>(s) + (q ? tail_step(s) : 0); }
     __device__ static void vec_words(const uint32_t (&w)[6], Vec &v)
     {
@@ -539,15 +535,6 @@ template <> struct Prec<HISQ_F64X> {
     struct Vec { float h[6], l[6]; };
     struct Acc { DAcc v[6]; };
     static constexpr int SB = 48;
-    __device__ static size_t chunk_off(uint32_t s, int q) { return blocked_off<SB>(s) + 512 * q; }
-    __device__ static void vec_words(const uint32_t (&w)[12], Vec &v)
-    {
-#pragma unroll
-        for (int i = 0; i < 6; i++) {
-            v.h[i] = __uint_as_float(w[i]);
-            v.l[i] = __uint_as_float(w[6 + i]);
-        }
-    }
     template <int NREAL>
     __device__ static void unpack(const uint32_t *w, Link &U)
     {

@@ -49,14 +49,14 @@ struct PhaseSlot {
 static_assert(sizeof(PhaseSlot) == 64, "one arrival record per 64-byte line");
 static_assert(offsetof(PhaseSlot, part) % 16 == 0, "partial sums are read as 16-byte pairs");
 constexpr int kPhaseMaxBlocks = 1024;
-// shared memory per owned site: x, r, p, Ap (FP32 records)
+// shared memory per owned site: x, r, p, Ap (FP32 vectors in blocks of 32 sites, 24 bytes a site)
 constexpr int kPhaseSmemPerSite = 4 * 24;
 constexpr int kPhaseMaxSmem = 200 * 1024;
 
 struct PhaseArgs {
     DslashArgs doe;       // t = D_oe p   (output parity 1; in = p, out = t)
     DslashArgs deo;       // Ap = m4 p - D_eo t (output parity 0; in = t, m4)
-    char *x, *p, *r;      // FP32 iteration vectors (24-byte records) in global memory
+    char *x, *p, *r;      // FP32 iteration vectors (blocks of 32 sites) in global memory
     uint32_t Vh;
     uint32_t chunk;       // sites per block (multiple of 32)
     Scalars *sc;          // scalars of the right-hand side: read at entry, written at exit

@@ -17,7 +17,8 @@
 //     t when Nt < Nz shrinks that reuse distance, and with it the L2 footprint that keeps
 //     neighbour spinors of many right-hand sides resident.  Link stores too large for L2
 //     are then read with an evict-first policy so that the streamed links do not displace
-//     the spinors.
+//     the spinors, where links go through registers; copies to shared memory (PipeShape)
+//     take the ordinary priority.
 //   * DS threads per site (1, 2 or 4), each taking 4/DS of the directions; the partial sums
 //     meet through warp shuffles.  On small lattices one thread per site leaves a single
 //     short wave whose duration is the latency of 16 dependent gathers; splitting the
@@ -485,78 +486,78 @@ __device__ __forceinline__ void dslash_item(const DslashArgs &a, const Geom &g, 
             }
         } else {
 #pragma unroll
-        for (int m = 0; m < NMU; m++) {
-            const int mu = part * NMU + m;
-            typename T::Acc dacc[SPLIT ? NR : 1];
-            if constexpr (SPLIT) {
+            for (int m = 0; m < NMU; m++) {
+                const int mu = part * NMU + m;
+                typename T::Acc dacc[SPLIT ? NR : 1];
+                if constexpr (SPLIT) {
 #pragma unroll
-                for (int r = 0; r < NR; r++) T::zero(dacc[r]);
-            }
-            if constexpr (PF) {
-                // the loads of all four hops first (8 to 12 independent requests per thread in
-                // flight at once), then their products
-                uint32_t w[4][LB / 4];
-                typename T::Vec v[4][NR];
-                bool wrap[4];
-#pragma unroll
-                for (int h = 0; h < 4; h++) {
-                    const int k = h == 0 ? 1 : h == 1 ? -1 : h == 2 ? 3 : -3;
-                    const int type = h >> 1;
-                    const bool back = h & 1;
-                    const uint32_t sn = neighbour(g, c, s, mu, k, wrap[h]);
-                    const int lp = back ? 1 - a.p : a.p;
-                    const char *slot = links + (size_t)((lp * 2 + type) * 4 + mu) * slot_bytes;
-                    load_link_words<LB, LL1>(slot, back ? sn : s, w[h], NR > 1 && a.stream_links != 0);
-#pragma unroll
-                    for (int r = 0; r < NR; r++) vec_load<T, COH>(in + (size_t)r * a.rhs_bytes, sn, v[h][r]);
+                    for (int r = 0; r < NR; r++) T::zero(dacc[r]);
                 }
+                if constexpr (PF) {
+                    // the loads of all four hops first (8 to 12 independent requests per thread in
+                    // flight at once), then their products
+                    uint32_t w[4][LB / 4];
+                    typename T::Vec v[4][NR];
+                    bool wrap[4];
 #pragma unroll
-                for (int h = 0; h < 4; h++) {
-                    const int type = h >> 1;
-                    const bool back = h & 1;
-                    typename T::Link U;
-                    TL::template unpack<NREAL>(w[h], U);
-                    if constexpr (NREAL == 12) T::rebuild(U, (eta_neg(c, mu) != 0) ^ (mu == 3 && wrap[h]));
+                    for (int h = 0; h < 4; h++) {
+                        const int k = h == 0 ? 1 : h == 1 ? -1 : h == 2 ? 3 : -3;
+                        const int type = h >> 1;
+                        const bool back = h & 1;
+                        const uint32_t sn = neighbour(g, c, s, mu, k, wrap[h]);
+                        const int lp = back ? 1 - a.p : a.p;
+                        const char *slot = links + (size_t)((lp * 2 + type) * 4 + mu) * slot_bytes;
+                        load_link_words<LB, LL1>(slot, back ? sn : s, w[h], NR > 1 && a.stream_links != 0);
 #pragma unroll
-                    for (int r = 0; r < NR; r++) {
-                        typename T::Acc &dst = SPLIT ? dacc[SPLIT ? r : 0] : acc[TWO ? type : 0][r];
-                        if (back) T::template hop<true, true>(dst, U, v[h][r]);
-                        else T::template hop<false, false>(dst, U, v[h][r]);
+                        for (int r = 0; r < NR; r++) vec_load<T, COH>(in + (size_t)r * a.rhs_bytes, sn, v[h][r]);
+                    }
+#pragma unroll
+                    for (int h = 0; h < 4; h++) {
+                        const int type = h >> 1;
+                        const bool back = h & 1;
+                        typename T::Link U;
+                        TL::template unpack<NREAL>(w[h], U);
+                        if constexpr (NREAL == 12) T::rebuild(U, (eta_neg(c, mu) != 0) ^ (mu == 3 && wrap[h]));
+#pragma unroll
+                        for (int r = 0; r < NR; r++) {
+                            typename T::Acc &dst = SPLIT ? dacc[SPLIT ? r : 0] : acc[TWO ? type : 0][r];
+                            if (back) T::template hop<true, true>(dst, U, v[h][r]);
+                            else T::template hop<false, false>(dst, U, v[h][r]);
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int h = 0; h < 4; h++) {
+                        const int k = h == 0 ? 1 : h == 1 ? -1 : h == 2 ? 3 : -3;
+                        const int type = h >> 1;
+                        const bool back = h & 1;
+                        bool wrap;
+                        const uint32_t sn = neighbour(g, c, s, mu, k, wrap);
+                        const int lp = back ? 1 - a.p : a.p;
+                        const char *slot = links + (size_t)((lp * 2 + type) * 4 + mu) * slot_bytes;
+                        uint32_t w[LB / 4];
+                        load_link_words<LB, LL1>(slot, back ? sn : s, w, NR > 1 && a.stream_links != 0);
+                        typename T::Link U;
+                        TL::template unpack<NREAL>(w, U);
+                        if constexpr (NREAL == 12) T::rebuild(U, (eta_neg(c, mu) != 0) ^ (mu == 3 && wrap));
+#pragma unroll
+                        for (int r = 0; r < NR; r++) {
+                            typename T::Vec v;
+                            vec_load<T, COH>(in + (size_t)r * a.rhs_bytes, sn, v);
+                            typename T::Acc &dst = SPLIT ? dacc[SPLIT ? r : 0] : acc[TWO ? type : 0][r];
+                            if (back) T::template hop<true, true>(dst, U, v);
+                            else T::template hop<false, false>(dst, U, v);
+                        }
                     }
                 }
-            } else {
+                if constexpr (SPLIT) {
 #pragma unroll
-            for (int h = 0; h < 4; h++) {
-                const int k = h == 0 ? 1 : h == 1 ? -1 : h == 2 ? 3 : -3;
-                const int type = h >> 1;
-                const bool back = h & 1;
-                bool wrap;
-                const uint32_t sn = neighbour(g, c, s, mu, k, wrap);
-                const int lp = back ? 1 - a.p : a.p;
-                const char *slot = links + (size_t)((lp * 2 + type) * 4 + mu) * slot_bytes;
-                uint32_t w[LB / 4];
-                load_link_words<LB, LL1>(slot, back ? sn : s, w, NR > 1 && a.stream_links != 0);
-                typename T::Link U;
-                TL::template unpack<NREAL>(w, U);
-                if constexpr (NREAL == 12) T::rebuild(U, (eta_neg(c, mu) != 0) ^ (mu == 3 && wrap));
-#pragma unroll
-                for (int r = 0; r < NR; r++) {
-                    typename T::Vec v;
-                    vec_load<T, COH>(in + (size_t)r * a.rhs_bytes, sn, v);
-                    typename T::Acc &dst = SPLIT ? dacc[SPLIT ? r : 0] : acc[TWO ? type : 0][r];
-                    if (back) T::template hop<true, true>(dst, U, v);
-                    else T::template hop<false, false>(dst, U, v);
+                    for (int r = 0; r < NR; r++) {
+                        if (m == 0) acc[0][r] = dacc[r];
+                        else T::add_acc(acc[0][r], dacc[r]);
+                    }
                 }
             }
-            }
-            if constexpr (SPLIT) {
-#pragma unroll
-                for (int r = 0; r < NR; r++) {
-                    if (m == 0) acc[0][r] = dacc[r];
-                    else T::add_acc(acc[0][r], dacc[r]);
-                }
-            }
-        }
         }
 #pragma unroll
         for (int r = 0; r < NR; r++) {
