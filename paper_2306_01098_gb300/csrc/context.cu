@@ -109,13 +109,21 @@ __global__ void k_import_links(const ImportArgs a)
         const size_t V = 2ull * a.g.Vh;
         const double *L = a.src[type] + ((size_t)mu * V + (size_t)p * a.g.Vh + s) * 18;
         if (a.fixed) {
+            // words of its own, taken by constant numbers, stay in registers (w, which the other precisions fill by
+            // running numbers, is in local memory: 1 ms more on 32^3 x 8, where a context with FP64 links takes 2.0)
             double d[18];
+            uint32_t f[36];
+            uint64_t rest;
 #pragma unroll
             for (int i = 0; i < 18; i++) d[i] = sg * L[i];
-            uint64_t rest;
-            fx_encode_link(d, w, rest);
-            reinterpret_cast<uint64_t *>(dst + (size_t)a.g.VhPad * LB)[s] = rest;
-        } else for (int i = 0; i < a.nreal; i++) {
+            fx_encode_link(d, f, rest);
+            uint4 *q = reinterpret_cast<uint4 *>(dst + (size_t)(s >> 5) * (32 * 144)) + (s & 31);
+#pragma unroll
+            for (int k = 0; k < 9; k++) q[32 * k] = make_uint4(f[4 * k], f[4 * k + 1], f[4 * k + 2], f[4 * k + 3]);
+            reinterpret_cast<uint64_t *>(dst + (size_t)a.g.VhPad * 144)[s] = rest;
+            return;
+        }
+        for (int i = 0; i < a.nreal; i++) {
             const double d = sg * L[i];
             switch (a.prec) {
             case HISQ_F64: {
