@@ -26,8 +26,9 @@
 //   * Links (PL) stream through with L1-bypassing 16-byte loads, read once per application;
 //     neighbour spinors (PV) are gathered through L1/L2, where their 16-fold reuse happens.
 //     PL and PV differ only for 16-bit links with FP32 vectors.
-//   * FP64 with 18 reals runs on integers (fixed.cuh), 1.9 times as fast as FP64 multiply-adds on
-//     this GPU and no less precise; 12 reals stay in FP64 (their third row is rebuilt in it).
+//   * FP64 with 18 reals runs on integers (fixed.cuh), twice as fast as FP64 multiply-adds on
+//     this GPU; sites whose components would be less precise than theirs go to FP64.  12 reals stay in
+//     FP64 (their third row is rebuilt in it).
 // Optional epilogue (normal operator, Sec. 3.2 applyMdaggM):
 //   EPI = 1: out = m4 * p - D in,   and <p, out> reduced in FP64 per right-hand side;
 //   EPI = 2: the same and also |r|^2, <r, out> and <out, out> (four values per right-hand
@@ -136,8 +137,8 @@ __device__ __forceinline__ void vec_load(const char *base, uint32_t s, typename 
 // the requests in flight cost no registers and nothing keeps a warp from running ahead.  No thread
 // reads another's part: the only waits are the thread's own (cp.async groups, one per hop).
 // Used where registers limit the warps in flight: the fixed-point FP64 sites (a hop's link is 36
-// registers; 137 -> 131 us for the 32^3 x 8 normal operator, 905 -> 853 us for a 64^3 x 16 Dslash,
-// 0.87 of the HBM rate) and FP32 vectors with four or more right-hand sides a thread (or two, with
+// registers; 137 -> 131 us for the 32^3 x 8 normal operator, 905 -> 853 us for a 64^3 x 16 Dslash, both
+// before their sums were held to FP64 component by component: 137 and 920 us now) and FP32 vectors with four or more right-hand sides a thread (or two, with
 // the third rows of 12-real links to rebuild): 32^3 x 16, 16-bit links, 8 right-hand sides, 159 -> 142 ms
 // a solve.  With one or two right-hand sides of 18-real links the extra trip costs more than the
 // registers do (FP32 64^3 x 16 467 -> 479 us, float pairs 18 x 22 x 14 x 10, three sides, 83 -> 94 us).

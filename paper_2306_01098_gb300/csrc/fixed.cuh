@@ -27,7 +27,8 @@
 // point or wall source.
 // Measured (max over a field, relative to its largest entry): 2.4e-16 after the normal operator of a
 // 32^3 x 8 lattice, 3.9e-16 with FP64 multiply-adds.  Time there, two Dslash launches: 280.8 us with
-// FP64 multiply-adds (their pipe alone needs 250 us), 131 us so (the bytes need 93 us).
+// FP64 multiply-adds (their pipe alone needs 250 us), 130 us in fixed point without a look at the components, 137 us so
+// (the bytes need 93 us).
 // Sites that meet anything this cannot hold (an infinity or NaN, a link or vector whose largest real is
 // below about 1e-289, products outside about 1e-254 .. 1e287, a link whose reals lie too far apart) are
 // computed in FP64 instead (fx_sites_f64), from the same doubles.

@@ -42,7 +42,7 @@ __device__ __forceinline__ uint32_t bf_pack(float a, float b)
 
 // the C channels of site i, 3 words each: as 16-byte loads where the records allow it (word by word
 // every load of a warp touches its sites' whole 24 or 12 cache lines; with the stores likewise, the
-// network on 32^3 x 8 takes 318 us instead of 366)
+// network on 32^3 x 8 takes 320 us instead of 368)
 template <int C>
 __device__ __forceinline__ void load_site(const uint32_t *act, uint32_t i, uint32_t (&w)[3 * C])
 {
@@ -479,7 +479,7 @@ __device__ __forceinline__ void warp_sums(float (&v)[NV])
 // per block row.  Per site and tap 36 FP32 operations per input channel transport it and 12 per pair of
 // channels multiply; the sums over a warp's sites cost 31 shuffles per 32 real values (warp_sums).
 // Two sums of five shuffles for each of the 64 pairs, one block for all taps, took 270 us for
-// 16^3 x 8 sites, 8 -> 8 channels (loss and gradient of the default network there: 936 us, 401 us now).
+// 16^3 x 8 sites, 8 -> 8 channels (loss and gradient of the default network there: 961 us, 423 us now).
 template <int PL, int CIN, int COUT>
 __global__ void __launch_bounds__(128) k_net_wgrad(const NetLayerArgs a, const uint32_t *gout, float2 *part)
 {

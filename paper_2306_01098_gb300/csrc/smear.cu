@@ -434,7 +434,7 @@ struct Coef {
 // issue at eight warps an SM (the operands of a product fill the registers).  One thread per (site,
 // detour) in launches 1 and 2, one per site in 3, consecutive sites in consecutive lanes.
 // 24^3 x 8, the whole call with projection and Naik links: 76.0 ms with every path multiplied out, 12.4
-// with stored staples in FP64, 7.6 with these products, 6.7 with the projection of now, 7.0 with the look at what
+// with stored staples in FP64, 7.6 with these products, 6.7 with the projection of now, 7.1 with the look at what
 // enters each entry (product).
 __global__ void __launch_bounds__(128) k_stap3(Lat L, const double2 *u, int mu, double2 *t, double2 *td)
 {
